@@ -1,6 +1,9 @@
 // Accept / reject, step-size adaptation, thinning and pooling (Algorithm 2,
 // Eq. BME2), the diagnostics reductions (Eq. ACFrho, Eq. IACT) and small test hooks.
 #include "qst_internal.cuh"
+#include "f32x2.cuh"
+
+#include <atomic>
 
 namespace qst {
 namespace {
@@ -203,45 +206,164 @@ __global__ void __launch_bounds__(32 * kReduceWarps) pool_reduce_kernel(const do
     }
 }
 
-// Eq. ACFrho for one diagnostic chain per CTA: c~[l] = sum_{n < N - lmax} sum_e w_e
-// (x_n,e - m_e)(x_{n+l},e - m_e) with w_e = 1 on the diagonal and 2 off it (each packed
-// off-diagonal entry stands for the (i,j) and (j,i) terms of Eq. ACFa).  Products in
-// FP32 summed over chunks of 32 samples, chunks accumulated in FP64.
-__global__ void acf_kernel(const float *traj, int traj_cap, int d, int D, int n_kept, int lmax, double *out) {
-    extern __shared__ float sh[];  // mean[d]
-    __shared__ double red[kThreads];
-    const float *x = traj + (int64_t)blockIdx.x * traj_cap * d;
-    for (int e = threadIdx.x; e < d; e += blockDim.x) {
-        double s = 0.0;
-        for (int n = 0; n < n_kept; ++n) s += x[(int64_t)n * d + e];
-        sh[e] = (float)(s / n_kept);
-    }
-    __syncthreads();
-    const int m = n_kept - lmax;
-    for (int l = 0; l <= lmax; ++l) {
-        double acc = 0.0;
-        for (int e = threadIdx.x; e < d; e += blockDim.x) {
-            const float mu = sh[e];
-            const float w = ((e / D) == (e % D)) ? 1.0f : 2.0f;
-            float chunk = 0.0f;
-            for (int n = 0; n < m; ++n) {
-                chunk = __fmaf_rn(x[(int64_t)n * d + e] - mu, x[(int64_t)(n + l) * d + e] - mu, chunk);
-                if ((n & 31) == 31) {
-                    acc += (double)(w * chunk);
-                    chunk = 0.0f;
+// Eq. ACFrho of the diagnostic chains: c~[l] = sum_{n < N - lmax} sum_e w_e (x_n,e - m_e)
+// (x_{n+l},e - m_e) with w_e = 1 on the diagonal and 2 off it (each packed off-diagonal entry
+// stands for the (i,j) and (j,i) terms of Eq. ACFa).  Products in FP32 summed over chunks of 32
+// samples; chunks, entries and slabs are added as exact FP32 pairs and in FP64.
+//
+// The work is d (N - lmax) (lmax + 1) multiply-adds per chain on N d values, so it is bound by
+// the FP32 pipe once each value is loaded rarely enough.  A CTA takes one chain, a slab of up to
+// kAcfEntries packed entries and kAcfLags lags.  A thread owns a pair of entries (f32x2) and
+// kAcfTile consecutive lags: the centred samples sit in shared memory, and a register window of
+// kAcfTile samples slides along, so two 64-bit loads feed kAcfTile packed FMAs (one load per FMA
+// operand, one entry and one lag at a time, took 12.8 ms for 256 four-qubit chains of 600 states
+// and 201 lags; this form 0.41 ms, the FP32 pipe busy half of it).  Samples pass through in segments of kAcfSeg, so neither N
+// nor lmax is limited by shared memory.
+constexpr int kAcfEntries = 32;                          // packed entries per slab
+constexpr int kAcfTile = 16;                             // lags per thread
+constexpr int kAcfLagTiles = 13;                         // lag tiles per CTA (l_max = 200 fits one CTA)
+constexpr int kAcfLags = kAcfTile * kAcfLagTiles;        // 208
+constexpr int kAcfSeg = 256;                             // samples n per segment (a multiple of 32)
+constexpr int kAcfRowsB = kAcfSeg + kAcfLags;            // samples n + l of a segment
+constexpr int kAcfThreads = kAcfEntries / 2 * kAcfLagTiles;   // 208
+constexpr size_t kAcfSmem = sizeof(float) * kAcfEntries * (kAcfSeg + kAcfRowsB);
+
+// part[chain][slab][l]: the slab's share of c~[l]; grid (chains, slabs, lag groups)
+__global__ void __launch_bounds__(kAcfThreads, 2) acf_kernel(const float *traj, int traj_cap, int d, int D, int n_kept,
+                                                          int lmax, double *part) {
+    extern __shared__ __align__(16) float acf_sm[];
+    float *za = acf_sm, *zb = acf_sm + kAcfSeg * kAcfEntries;   // [sample][entry], centred
+    __shared__ __align__(16) float mean[kAcfEntries];
+    const int ne = min(kAcfEntries, d);                 // entries of a slab (d is 4, 16 or a multiple of 32)
+    const int np = ne / 2;                              // entry pairs: consecutive lanes
+    const int tid = threadIdx.x;
+    const int pr = tid % np, lt = tid / np;             // this thread's pair and lag tile
+    const bool worker = lt < kAcfLagTiles;
+    const int e0 = blockIdx.y * ne;
+    const float *x = traj + (int64_t)blockIdx.x * traj_cap * d + e0;
+
+    // means over all N samples: exact pairs per thread, joined in FP64
+    {
+        float2 hi = make_float2(0.f, 0.f), lo = hi;
+        const int lanes = kAcfThreads / np;
+        constexpr int kInFlight = 16;   // loads requested together (one at a time: half of the kernel's time)
+        if (lt < lanes)
+            for (int n = lt; n < n_kept; n += kInFlight * lanes) {
+                float2 v[kInFlight];
+#pragma unroll
+                for (int u = 0; u < kInFlight; ++u) {
+                    v[u] = make_float2(0.f, 0.f);
+                    if (n + u * lanes < n_kept)
+                        v[u] = *reinterpret_cast<const float2 *>(x + (int64_t)(n + u * lanes) * d + 2 * pr);
+                }
+#pragma unroll
+                for (int u = 0; u < kInFlight; ++u) {
+                    float e;
+                    two_sum(hi.x, v[u].x, hi.x, e);
+                    lo.x += e;
+                    two_sum(hi.y, v[u].y, hi.y, e);
+                    lo.y += e;
                 }
             }
-            acc += (double)(w * chunk);
+        double *md = reinterpret_cast<double *>(acf_sm);   // [lane][entry] sums, before the samples move in
+        if (lt < lanes) {
+            md[lt * ne + 2 * pr] = (double)hi.x + (double)lo.x;
+            md[lt * ne + 2 * pr + 1] = (double)hi.y + (double)lo.y;
         }
-        red[threadIdx.x] = acc;
         __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-            __syncthreads();
+        if (tid < ne) {
+            double s = 0.0;
+            for (int q = 0; q < lanes; ++q) s += md[q * ne + tid];
+            mean[tid] = (float)(s / n_kept);
         }
-        if (threadIdx.x == 0) out[(int64_t)blockIdx.x * (lmax + 1) + l] = red[0];
         __syncthreads();
     }
+
+    const int m = n_kept - lmax;
+    const int l0 = blockIdx.z * kAcfLags;              // this CTA's lags l0 .. l0 + kAcfLags - 1
+    const int lag = lt * kAcfTile;
+    const int ea = e0 + 2 * pr;
+    const int nq = ne / 4, lq = tid % nq, lr = tid / nq;   // loads: this thread's float4 column (208 is a multiple of nq)
+    const float4 mq = *reinterpret_cast<const float4 *>(mean + 4 * lq);
+    const float2 w = make_float2((ea / D) == (ea % D) ? 1.0f : 2.0f, ((ea + 1) / D) == ((ea + 1) % D) ? 1.0f : 2.0f);
+    float hi[kAcfTile], lo[kAcfTile];   // sums over both entries
+#pragma unroll
+    for (int i = 0; i < kAcfTile; ++i) hi[i] = lo[i] = 0.0f;
+    for (int n0 = 0; n0 < m; n0 += kAcfSeg) {
+        const int rows = min(kAcfSeg, (m - n0 + 31) / 32 * 32);   // whole chunks; samples n >= m count as zero
+        __syncthreads();
+        // the first lag group's samples n are the first rows of its samples n + l: only later
+        // groups, and a segment that ends at m (samples from there on count as zero), load them apart
+        auto fill = [&](float *z, int first, int count, int end) {
+#pragma unroll 4
+            for (int r = lr; r < count; r += kAcfThreads / nq) {
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (first + r < end) {
+                    v = *reinterpret_cast<const float4 *>(x + (int64_t)(first + r) * d + 4 * lq);
+                    v = make_float4(v.x - mq.x, v.y - mq.y, v.z - mq.z, v.w - mq.w);
+                }
+                *reinterpret_cast<float4 *>(z + r * ne + 4 * lq) = v;
+            }
+        };
+        const bool own = l0 != 0 || n0 + rows > m;
+        if (own) fill(za, n0, rows, m);
+        fill(zb, n0 + l0, rows + kAcfLags, n_kept);
+        __syncthreads();
+        if (worker) {
+            const float *pa = (own ? za : zb) + 2 * pr, *pb = zb + lag * ne + 2 * pr;
+            float2 win[kAcfTile];   // sample n + lag + i in slot (n + i) mod kAcfTile
+#pragma unroll
+            for (int i = 0; i < kAcfTile; ++i) win[i] = *reinterpret_cast<const float2 *>(pb + i * ne);
+            float2 a_next = *reinterpret_cast<const float2 *>(pa);
+#pragma unroll 1
+            for (int c = 0; c < rows; c += 32) {
+                float2 chunk[kAcfTile];
+#pragma unroll
+                for (int i = 0; i < kAcfTile; ++i) chunk[i] = make_float2(0.f, 0.f);
+#pragma unroll 1
+                for (int h = c; h < c + 32; h += kAcfTile) {
+#pragma unroll
+                    for (int u = 0; u < kAcfTile; ++u) {
+                        const float2 a = a_next;   // (the row after the last one is zb's first)
+                        a_next = *reinterpret_cast<const float2 *>(pa + (h + u + 1) * ne);
+#pragma unroll
+                        for (int i = 0; i < kAcfTile; ++i)
+                            chunk[i] = fma2(a, win[(u + i) % kAcfTile], chunk[i]);
+                        // the sample kAcfTile further on (the last row read is rows + kAcfTile - 1 past the tile)
+                        win[u] = *reinterpret_cast<const float2 *>(pb + (h + u + kAcfTile) * ne);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < kAcfTile; ++i) {   // hi + lo += w chunk, exactly (two-sum)
+                    const float2 v = mul2(w, chunk[i]);
+                    float e, e2;
+                    two_sum(hi[i], v.x, hi[i], e);
+                    two_sum(hi[i], v.y, hi[i], e2);
+                    lo[i] += e + e2;
+                }
+            }
+        }
+    }
+    // the pairs of a lag tile sit in np consecutive lanes (a power of two, 2 .. 16): FP64 tree
+    double *out = part + ((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * (lmax + 1);
+    const unsigned lanes_mask = (tid / 32 + 1) * 32 <= kAcfThreads ? 0xffffffffu : (1u << (kAcfThreads % 32)) - 1u;
+#pragma unroll
+    for (int i = 0; i < kAcfTile; ++i) {
+        double v = (double)hi[i] + (double)lo[i];
+        for (int off = np / 2; off > 0; off >>= 1) v += __shfl_xor_sync(lanes_mask, v, off);
+        const int l = l0 + lag + i;
+        if (worker && pr == 0 && l <= lmax) out[l] = v;
+    }
+}
+
+// out[chain][l] = sum over the slabs, in slab order
+__global__ void acf_reduce_kernel(const double *part, int slabs, int nl, int64_t total, double *out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= total) return;
+    const int64_t c = i / nl, l = i - c * nl;
+    double s = 0.0;
+    for (int b = 0; b < slabs; ++b) s += part[(c * slabs + b) * nl + l];
+    out[i] = s;
 }
 
 // log L = C0 - N log t + sum over column groups, for stateless evaluation.
@@ -327,9 +449,29 @@ cudaError_t launch_pool_reduce(const ProblemView &p, double *out, cudaStream_t s
     return cudaGetLastError();
 }
 
-cudaError_t launch_acf(const ProblemView &p, int n_kept, int lmax, double *acf_raw, cudaStream_t s) {
+int acf_slabs(int d) { return (d + kAcfEntries - 1) / kAcfEntries; }
+
+cudaError_t launch_acf(const ProblemView &p, int n_kept, int lmax, double *part, cudaStream_t s) {
     if (p.n_diag <= 0 || n_kept <= lmax) return cudaSuccess;
-    acf_kernel<<<p.n_diag, kThreads, sizeof(float) * p.d, s>>>(p.traj, p.traj_cap, p.d, p.D, n_kept, lmax, acf_raw);
+    // more than 48 KB of dynamic shared memory: opted into once per device
+    static std::atomic<unsigned long long> attr_set{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !((attr_set.load() >> dev) & 1ull)) {
+        e = cudaFuncSetAttribute(acf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAcfSmem);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) attr_set.fetch_or(1ull << dev);
+    }
+    const int slabs = acf_slabs(p.d);
+    const dim3 grid((unsigned)p.n_diag, (unsigned)slabs, (unsigned)(lmax / kAcfLags + 1));
+    acf_kernel<<<grid, kAcfThreads, kAcfSmem, s>>>(p.traj, p.traj_cap, p.d, p.D, n_kept, lmax, part);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_acf_reduce(const ProblemView &p, int lmax, const double *part, double *acf_raw, cudaStream_t s) {
+    const int64_t total = (int64_t)p.n_diag * (lmax + 1);
+    acf_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(part, acf_slabs(p.d), lmax + 1, total, acf_raw);
     return cudaGetLastError();
 }
 

@@ -122,6 +122,7 @@ struct Plan {
     std::vector<HostProblem> probs;
     size_t status_off = 0;  // device status word
     size_t step_off = 0;    // device StepState
+    size_t acf_part_off = 0;   // the ACF's partial sums (one problem's at a time; not chain state)
     size_t bytes = 0;       // total workspace bytes
 };
 
@@ -517,6 +518,11 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
     }
     plan.status_off = take(256);
     plan.step_off = take(256);
+    size_t acf_part = 0;
+    for (const auto &hp : plan.probs)
+        if (hp.v.n_diag > 0 && hp.v.traj_cap > cfg->acf_lmax)
+            acf_part = std::max(acf_part, sizeof(double) * (size_t)hp.v.n_diag * acf_slabs(hp.v.d) * (cfg->acf_lmax + 1));
+    plan.acf_part_off = take(acf_part);
     plan.bytes = off;
     return QST_OK;
 }
@@ -1161,7 +1167,11 @@ qst_status qst_diagnostics(qst_handle *h, int32_t problem, qst_diag *out, double
     std::vector<double> raw;
     if (do_acf) {
         double *acf_dev = reinterpret_cast<double *>(h->ws + hp->off.acf);
-        st = launch(h, QST_KERNEL_DIAG, "acf", [&] { return launch_acf(v, n_kept, lmax, acf_dev, h->stream); });
+        double *part = reinterpret_cast<double *>(h->ws + h->plan.acf_part_off);
+        st = launch(h, QST_KERNEL_DIAG, "acf", [&] { return launch_acf(v, n_kept, lmax, part, h->stream); });
+        if (st != QST_OK) return st;
+        st = launch(h, QST_KERNEL_DIAG, "acf reduce",
+                    [&] { return launch_acf_reduce(v, lmax, part, acf_dev, h->stream); });
         if (st != QST_OK) return st;
         raw.resize((size_t)v.n_diag * (lmax + 1));
         QST_CUDA(cudaMemcpyAsync(raw.data(), acf_dev, sizeof(double) * raw.size(), cudaMemcpyDeviceToHost, h->stream),

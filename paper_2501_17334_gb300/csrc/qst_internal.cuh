@@ -198,7 +198,10 @@ cudaError_t launch_project_fp32(const ProblemView &p, const float *A, int64_t ro
 cudaError_t launch_accept(const ProblemView &p, const SamplerParams &sp, int mode, const StepState *step_dev, uint32_t step, bool kept,
                           int64_t kept_idx, uint32_t *status, cudaStream_t s);
 cudaError_t launch_pool_reduce(const ProblemView &p, double *out, cudaStream_t s);
-cudaError_t launch_acf(const ProblemView &p, int n_kept, int lmax, double *acf_raw, cudaStream_t s);
+// ACF sums of the diagnostic chains: part [n_diag][acf_slabs(d)][lmax + 1], then acf_raw [n_diag][lmax + 1]
+int acf_slabs(int d);
+cudaError_t launch_acf(const ProblemView &p, int n_kept, int lmax, double *part, cudaStream_t s);
+cudaError_t launch_acf_reduce(const ProblemView &p, int lmax, const double *part, double *acf_raw, cudaStream_t s);
 cudaError_t launch_logl_combine(const ProblemView &p, int64_t rows, double *out, cudaStream_t s);
 cudaError_t launch_philox_blocks(uint64_t seed, uint32_t step, uint32_t tag, uint32_t chain0, int64_t nchains,
                                  uint32_t block0, int32_t nblocks, uint32_t *out, cudaStream_t s);
