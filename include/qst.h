@@ -139,7 +139,8 @@ typedef struct {
                                qubits still take 2) */
     int32_t use_graph;      /* 1 (default): qst_run_chains replays one step captured as a CUDA graph
                                (the step counter lives on the device); 0: plain launches. Kernel
-                               timing (qst_set_profiling) always uses plain launches */
+                               timing (qst_set_profiling) always uses plain launches.  Problems that
+                               run many steps per launch (qst_run_chains) do so with either */
     int32_t autotune;       /* 1 (default): qst_create times, for every problem, the projection with
                                each candidate number of column groups (the split of its N tiles
                                over CTAs) and, at 1-4 qubits with fewer chains than fill the GPU
@@ -226,7 +227,11 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
  * proposal, projection and accept kernels of every problem.  With use_graph the first
  * call captures that sequence once (on private streams, the problems of a handle on up
  * to eight parallel branches, since they are independent) and every step launches the
- * graph; the results are bit-identical to plain launches.
+ * graph; the results are bit-identical to plain launches.  One- and two-qubit problems in the FP32
+ * or the structured Pauli form (up to 16 settings at two qubits, 8 at one, 2^18 / 4^(Q-1) chains,
+ * qr_passes 3 or the Hilbert-Schmidt prior) instead run many steps per launch, on their own
+ * branches beside the other problems, with the same results bit for bit; not while kernel timing
+ * is on (qst_set_profiling).
  * Errors: QST_ERR_INVALID_ARG if num_steps < 0. */
 qst_status qst_run_chains(qst_handle *h, int64_t num_steps);
 

@@ -116,12 +116,15 @@ struct HostProblem {
     std::vector<float2> pauli_wc;     // and counts
     std::vector<int32_t> pauli_perm;  // tree order -> setting-major projector index
     TcPlan *tc = nullptr;
+    size_t hist_off = 0;              // kept states of a multi-step launch (fused_small.cu)
 };
 
 struct Plan {
     std::vector<HostProblem> probs;
     size_t status_off = 0;  // device status word
     size_t step_off = 0;    // device StepState
+    size_t base_off = 0;    // device StepState: the counter before a qst_run_chains call (multi-step launches)
+    size_t clear_bytes = 0; // leading bytes that start as zeros
     size_t acf_part_off = 0;   // the ACF's partial sums (one problem's at a time; not chain state)
     size_t bytes = 0;       // total workspace bytes
 };
@@ -523,6 +526,10 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
         if (hp.v.n_diag > 0 && hp.v.traj_cap > cfg->acf_lmax)
             acf_part = std::max(acf_part, sizeof(double) * (size_t)hp.v.n_diag * acf_slabs(hp.v.d) * (cfg->acf_lmax + 1));
     plan.acf_part_off = take(acf_part);
+    plan.base_off = take(256);
+    plan.clear_bytes = off;   // what follows is written before it is read
+    for (auto &hp : plan.probs)
+        hp.hist_off = take(sizeof(float) * (size_t)fused_kept_steps(hp.v) * hp.v.R * hp.v.d);
     plan.bytes = off;
     return QST_OK;
 }
@@ -549,6 +556,7 @@ struct qst_handle {
     bool own_ws = false;
     uint32_t *d_status = nullptr;
     StepState *d_step = nullptr;
+    StepState *d_base = nullptr;
     cudaStream_t capture_stream = nullptr;   // private stream the step graph is captured on
     static constexpr int kBranches = 8;      // problems of a graph step run on up to 8 parallel branches
     cudaStream_t branch[kBranches] = {};
@@ -909,9 +917,10 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
         h->ws_bytes = h->plan.bytes;
         h->own_ws = true;
     }
-    QST_CUDA(cudaMemsetAsync(h->ws, 0, h->plan.bytes, h->stream), "clear workspace");
+    QST_CUDA(cudaMemsetAsync(h->ws, 0, h->plan.clear_bytes, h->stream), "clear workspace");
     h->d_status = reinterpret_cast<uint32_t *>(h->ws + h->plan.status_off);
     h->d_step = reinterpret_cast<StepState *>(h->ws + h->plan.step_off);
+    h->d_base = reinterpret_cast<StepState *>(h->ws + h->plan.base_off);
     for (auto &hp : h->plan.probs) {
         bind_problem(h.get(), hp);
         ProblemView &v = hp.v;
@@ -982,7 +991,8 @@ namespace {
 // One step's launches on h->stream: open step j on the device, then every problem's
 // proposal, projection and accept, all reading j from the device.  With `branches` (graph
 // capture) the problems are spread over parallel branches -- they are independent -- so
-// the graph runs the kernels of different problems concurrently.
+// the graph runs the kernels of different problems concurrently.  With `multi` the problems that
+// run many steps per launch (enqueue_multi) are left out.
 qst_status enqueue_problem(qst_handle *h, HostProblem &hp) {
     ProblemView &v = hp.v;
     qst_status st = launch(h, QST_KERNEL_PROPOSE, "propose", [&] {
@@ -996,14 +1006,17 @@ qst_status enqueue_problem(qst_handle *h, HostProblem &hp) {
     });
 }
 
-qst_status enqueue_step(qst_handle *h, bool branches) {
+qst_status enqueue_step(qst_handle *h, bool branches, bool multi) {
     qst_status st = launch(h, QST_KERNEL_ACCEPT, "advance step",
                            [&] { return launch_advance_step(h->d_step, h->cfg.thin, h->cfg.burn_in, h->stream); });
     if (st != QST_OK) return st;
-    const int np = (int)h->plan.probs.size();
+    std::vector<HostProblem *> probs;
+    for (auto &hp : h->plan.probs)
+        if (!multi || !fused_supported(hp.v)) probs.push_back(&hp);
+    const int np = (int)probs.size();
     if (!branches || np == 1) {
-        for (auto &hp : h->plan.probs) {
-            st = enqueue_problem(h, hp);
+        for (HostProblem *hp : probs) {
+            st = enqueue_problem(h, *hp);
             if (st != QST_OK) return st;
         }
         return QST_OK;
@@ -1014,7 +1027,7 @@ qst_status enqueue_step(qst_handle *h, bool branches) {
     for (int b = 0; b < nb; ++b) QST_CUDA(cudaStreamWaitEvent(h->branch[b], h->fork_ev, 0), "branch wait");
     for (int i = 0; i < np && st == QST_OK; ++i) {
         h->stream = h->branch[i % nb];
-        st = enqueue_problem(h, h->plan.probs[i]);
+        st = enqueue_problem(h, *probs[i]);
     }
     h->stream = origin;
     if (st != QST_OK) return st;
@@ -1025,22 +1038,48 @@ qst_status enqueue_step(qst_handle *h, bool branches) {
     return QST_OK;
 }
 
+// num_steps steps of one small problem on `s`: launches of up to 1024 steps (a few milliseconds
+// each) whose kept states fit the history buffer, each followed by their pooling.
+qst_status enqueue_multi(qst_handle *h, HostProblem &hp, int64_t num_steps, cudaStream_t s) {
+    const int thin = h->cfg.thin;
+    const int64_t burn = h->cfg.burn_in;
+    const int64_t most = std::min<int64_t>(1024, (int64_t)fused_kept_steps(hp.v) * thin);
+    float *hist = reinterpret_cast<float *>(h->ws + hp.hist_off);
+    for (int64_t off = 0; off < num_steps; off += most) {
+        const int n = (int)std::min<int64_t>(most, num_steps - off);
+        qst_status st = launch(h, QST_KERNEL_PROPOSE, "steps", [&] {
+            return launch_fused_steps(hp.v, h->sp, h->d_base, (uint32_t)off, n, thin, burn, hist, s);
+        });
+        if (st != QST_OK) return st;
+        st = launch(h, QST_KERNEL_ACCEPT, "pool steps", [&] {
+            return launch_fused_pool(hp.v, h->d_base, (uint32_t)off, n, thin, burn, hist, s);
+        });
+        if (st != QST_OK) return st;
+    }
+    return QST_OK;
+}
+
+qst_status create_branches(qst_handle *h) {
+    if (h->capture_stream) return QST_OK;
+    QST_CUDA(cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming), "create event");
+    for (int b = 0; b < qst_handle::kBranches; ++b) {
+        QST_CUDA(cudaStreamCreateWithFlags(&h->branch[b], cudaStreamNonBlocking), "create branch stream");
+        QST_CUDA(cudaEventCreateWithFlags(&h->join_ev[b], cudaEventDisableTiming), "create event");
+    }
+    QST_CUDA(cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking), "create capture stream");
+    return QST_OK;
+}
+
 // Captures enqueue_step once on the private capture stream and instantiates it.
 qst_status build_step_graph(qst_handle *h) {
-    if (!h->capture_stream) {
-        QST_CUDA(cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking), "create capture stream");
-        for (int b = 0; b < qst_handle::kBranches; ++b) {
-            QST_CUDA(cudaStreamCreateWithFlags(&h->branch[b], cudaStreamNonBlocking), "create branch stream");
-            QST_CUDA(cudaEventCreateWithFlags(&h->join_ev[b], cudaEventDisableTiming), "create event");
-        }
-        QST_CUDA(cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming), "create event");
-    }
+    const qst_status made = create_branches(h);
+    if (made != QST_OK) return made;
     cudaStream_t user = h->stream;
     const int64_t launches0 = h->launches;
     h->stream = h->capture_stream;
     cudaError_t e = cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal);
     qst_status st = QST_OK;
-    if (e == cudaSuccess) st = enqueue_step(h, true);
+    if (e == cudaSuccess) st = enqueue_step(h, true, true);
     cudaGraph_t g = nullptr;
     const cudaError_t e_end = (e == cudaSuccess) ? cudaStreamEndCapture(h->capture_stream, &g) : e;
     h->stream = user;
@@ -1063,9 +1102,32 @@ qst_status qst_run_chains(qst_handle *h, int64_t num_steps) {
     if (!h) return fail(QST_ERR_INVALID_ARG, "handle is NULL");
     if (num_steps < 0) return fail(QST_ERR_INVALID_ARG, "num_steps must be >= 0");
     if (h->steps_done + num_steps > 0xffffffffLL) return fail(QST_ERR_INVALID_ARG, "step counter exceeds 32 bits");
-    const bool graph = h->cfg.use_graph && !h->prof && num_steps > 0;
+    if (num_steps == 0) return QST_OK;
+    // problems that run many steps per launch (kernel timing takes the per-step kernels instead)
+    std::vector<HostProblem *> multi;
+    if (!h->prof)
+        for (auto &hp : h->plan.probs)
+            if (fused_supported(hp.v)) multi.push_back(&hp);
+    const bool steps = multi.size() < h->plan.probs.size();   // some problems go step by step
+    const bool graph = h->cfg.use_graph && !h->prof && steps;
     if (graph && !h->graph_exec) {
         qst_status st = build_step_graph(h);
+        if (st != QST_OK) return st;
+    }
+    int forked = 0;
+    if (!multi.empty()) {
+        qst_status st = launch(h, QST_KERNEL_ACCEPT, "snapshot step",
+                               [&] { return launch_snapshot_step(h->d_step, h->d_base, h->stream); });
+        if (st != QST_OK) return st;
+        if (steps || multi.size() > 1) {   // on their own branches, beside the other problems
+            st = create_branches(h);
+            if (st != QST_OK) return st;
+            forked = (int)std::min<size_t>(multi.size(), qst_handle::kBranches);
+            QST_CUDA(cudaEventRecord(h->fork_ev, h->stream), "fork");
+            for (int b = 0; b < forked; ++b) QST_CUDA(cudaStreamWaitEvent(h->branch[b], h->fork_ev, 0), "branch wait");
+        }
+        for (size_t i = 0; i < multi.size() && st == QST_OK; ++i)
+            st = enqueue_multi(h, *multi[i], num_steps, forked ? h->branch[i % forked] : h->stream);
         if (st != QST_OK) return st;
     }
     for (int64_t s = 0; s < num_steps; ++s) {
@@ -1074,12 +1136,22 @@ qst_status qst_run_chains(qst_handle *h, int64_t num_steps) {
         if (graph) {
             QST_CUDA(cudaGraphLaunch(h->graph_exec, h->stream), "launch step graph");
             h->launches += h->graph_kernels;
-        } else {
-            qst_status st = enqueue_step(h, false);
+        } else if (steps) {
+            qst_status st = enqueue_step(h, false, !h->prof);
             if (st != QST_OK) return st;
         }
         h->steps_done = j;
         if (kept) h->kept += 1;
+    }
+    if (!steps) {
+        qst_status st = launch(h, QST_KERNEL_ACCEPT, "advance steps", [&] {
+            return launch_advance_steps(h->d_step, (uint32_t)num_steps, h->cfg.thin, h->cfg.burn_in, h->stream);
+        });
+        if (st != QST_OK) return st;
+    }
+    for (int b = 0; b < forked; ++b) {
+        QST_CUDA(cudaEventRecord(h->join_ev[b], h->branch[b]), "join");
+        QST_CUDA(cudaStreamWaitEvent(h->stream, h->join_ev[b], 0), "join wait");
     }
     return QST_OK;
 }

@@ -207,6 +207,19 @@ cudaError_t launch_philox_blocks(uint64_t seed, uint32_t step, uint32_t tag, uin
                                  uint32_t block0, int32_t nblocks, uint32_t *out, cudaStream_t s);
 cudaError_t launch_inject_nan(const ProblemView &p, int64_t chain, cudaStream_t s);
 
+// Many steps of a one- or two-qubit problem in one launch (fused_small.cu).  `base`: the step counter
+// before the first launch of a qst_run_chains call, `off` the steps of its earlier launches; the
+// launch covers nsteps steps with at most fused_kept_steps(p) kept ones, whose states go to `hist`
+// ([kept step][R][d] floats) for launch_fused_pool.
+bool fused_supported(const ProblemView &p);
+int fused_kept_steps(const ProblemView &p);
+cudaError_t launch_fused_steps(const ProblemView &p, const SamplerParams &sp, const StepState *base, uint32_t off,
+                               int nsteps, int thin, int64_t burn_in, float *hist, cudaStream_t s);
+cudaError_t launch_fused_pool(const ProblemView &p, const StepState *base, uint32_t off, int nsteps, int thin,
+                              int64_t burn_in, const float *hist, cudaStream_t s);
+cudaError_t launch_snapshot_step(const StepState *st, StepState *base, cudaStream_t s);
+cudaError_t launch_advance_steps(StepState *st, uint32_t n, int thin, int64_t burn_in, cudaStream_t s);
+
 // tcgen05 projection in the view's tc_kind (sm_103a).  Returns cudaErrorNotSupported if the
 // shape is outside what the kernel handles.
 struct TcPlan;
