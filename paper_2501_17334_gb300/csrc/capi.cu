@@ -91,7 +91,7 @@ bool bf16_exact(double v) {
 // Per-problem host record and workspace layout
 // ------------------------------------------------------------------------------------------
 struct Layout {
-    size_t P32, Ptc, cnt, invf, ptot, colw, pauli_wq, pauli_wc, pauli_perm, y, cur, rho_cur, rho_prop, rho_split, trace_prop, logl_cur, logl_part, beta, coef,
+    size_t P32, sp_val, sp_code, sp_len, Ptc, cnt, invf, ptot, colw, pauli_wq, pauli_wc, pauli_perm, y, cur, rho_cur, rho_prop, rho_split, trace_prop, logl_cur, logl_part, beta, coef,
         acc_win,
         acc_total, pool, traj, trace_acc, trace_logl, red, acf, logl_eval, end;
 };
@@ -116,6 +116,7 @@ struct HostProblem {
     std::vector<float2> pauli_wc;     // and counts
     std::vector<int32_t> pauli_perm;  // tree order -> setting-major projector index
     TcPlan *tc = nullptr;
+    bool lists = false;               // the FP32 form's lists of used rows are kept (project_fp32.cu)
     size_t hist_off = 0;              // kept states of a multi-step launch (fused_small.cu)
 };
 
@@ -465,9 +466,13 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
             hp.group_choices = hp.tc_group_choices;
         } else {
             v.ngroups = fp32_ngroups(v, v.R);
-            const int nt = v.KD_pad / 128;
-            for (int g = 1; g < nt; g *= 2) hp.group_choices.push_back(g);
-            hp.group_choices.push_back(nt);
+            if (fp32_lists(v)) {   // an even share for every SM: nothing to tune
+                hp.group_choices = {v.ngroups};
+            } else {
+                const int nt = v.KD_pad / 128;
+                for (int g = 1; g < nt; g *= 2) hp.group_choices.push_back(g);
+                hp.group_choices.push_back(nt);
+            }
         }
         hp.part_slots = v.ngroups;
         for (int g : hp.group_choices) hp.part_slots = std::max(hp.part_slots, g);
@@ -490,6 +495,11 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
         Layout &L = hp.off;
         const int64_t R = v.R;
         L.P32 = take(sizeof(float) * hp.P32.size());
+        const bool lists = !tc && !hp.P32.empty() && fp32_lists(v);   // the FP32 form may run
+        L.sp_val = take(lists ? sizeof(float) * fp32_list_values(v) : 0);
+        L.sp_code = take(lists ? sizeof(uint32_t) * fp32_list_codes(v) : 0);
+        L.sp_len = take(lists ? sizeof(uint16_t) * fp32_list_lengths(v) : 0);
+        hp.lists = lists;
         L.Ptc = take(tc ? (size_t)tc_elem_bytes(kind) * v.KD_tc * v.d_pad : 0);
         L.cnt = take(sizeof(float) * hp.KDmax);
         L.invf = take(sizeof(float) * hp.KDmax);
@@ -628,6 +638,9 @@ qst_status bind_problem(qst_handle *h, HostProblem &hp) {
     ProblemView &v = hp.v;
     const Layout &L = hp.off;
     v.P32 = reinterpret_cast<const float *>(b + L.P32);
+    v.sp_val = hp.lists ? reinterpret_cast<const float *>(b + L.sp_val) : nullptr;
+    v.sp_code = reinterpret_cast<const uint32_t *>(b + L.sp_code);
+    v.sp_len = reinterpret_cast<const uint16_t *>(b + L.sp_len);
     v.Ptc = b + L.Ptc;
     v.cnt = reinterpret_cast<const float *>(b + L.cnt);
     v.invf = reinterpret_cast<const float *>(b + L.invf);
@@ -964,6 +977,12 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
         std::vector<float2> coef(v.R, make_float2((float)std::sqrt(1.0 - hp.beta0 * hp.beta0), (float)hp.beta0));
         QST_CUDA(cudaMemcpyAsync(v.coef, coef.data(), sizeof(float2) * v.R, cudaMemcpyHostToDevice, h->stream),
                  "upload proposal coefficients");
+        if (hp.lists) {
+            const cudaError_t e = launch_fp32_lists(v, v.P32, v.KD_pad, reinterpret_cast<float *>(h->ws + L.sp_val),
+                                                    reinterpret_cast<uint32_t *>(h->ws + L.sp_code),
+                                                    reinterpret_cast<uint16_t *>(h->ws + L.sp_len), h->stream);
+            if (e != cudaSuccess) return cuda_fail(e, "projector lists");
+        }
         // pageable copies above are staged synchronously; keep the host vectors alive until then
         QST_CUDA(cudaStreamSynchronize(h->stream), "stream sync");
         if (v.tc_kind != TC_NONE) {
@@ -1436,13 +1455,16 @@ qst_status qst_evaluate(qst_handle *h, int32_t problem, const float *x, int64_t 
         return launch_propose(v, MODE_EVAL, 0u, nullptr, x, n, uses_tc(v), rho, h->d_status, h->stream);
     });
     if (st != QST_OK) return st;
+    // a batch smaller than the chains: the FP32 form's CTAs may share its tiles more finely (as far as
+    // the partial sums' buffer goes)
+    const int groups = v.ngroups;
+    if (hp->lists)
+        v.ngroups = (int)std::max<int64_t>(1, std::min<int64_t>(fp32_ngroups(v, n), (int64_t)hp->part_slots * v.R / n));
     st = enqueue_projection(h, *hp, n, p);
-    if (st != QST_OK) return st;
-    if (logl) {
+    if (st == QST_OK && logl)
         st = launch(h, QST_KERNEL_DIAG, "logl combine", [&] { return launch_logl_combine(v, n, logl, h->stream); });
-        if (st != QST_OK) return st;
-    }
-    return QST_OK;
+    v.ngroups = groups;
+    return st;
 }
 
 qst_status qst_set_profiling(qst_handle *h, int32_t enabled) {

@@ -10,7 +10,8 @@
 // the whole device and stall every stream).  They pass their own inputs and outputs; the
 // library supplies the scratch.
 //
-// Scratch layout (bytes, all offsets 256-aligned): the padded projector matrix, the
+// Scratch layout (bytes, all offsets 256-aligned): the padded projector matrix (or, at three and
+// four qubits, the lists of its used rows), the
 // per-column weights and per-setting shot totals, the packed rho of every row, its trace, and the per-column-group
 // partial sums, for at most QST_NOALLOC_MAX_ROWS rows of at most 4 qubits.
 //
@@ -20,6 +21,7 @@
 // path waits for the device and no host buffer has to outlive the call.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 
@@ -43,6 +45,12 @@ constexpr size_t kOffRho = align256(kOffPtot + sizeof(float) * (kMaxKDPad / 2));
 constexpr size_t kOffTrace = align256(kOffRho + sizeof(float) * kMaxRows * kMaxDPad);
 constexpr size_t kOffPart = align256(kOffTrace + sizeof(double) * kMaxRows);
 constexpr size_t kScratchBytes = align256(kOffPart + sizeof(double) * kMaxGroups * kMaxRows);
+// the lists of used projector rows (three and four qubits) take the end of the partial sums
+constexpr int kListGroups = 7;
+constexpr size_t kOffCode = align256(kOffPart + sizeof(double) * kListGroups * kMaxRows);
+constexpr size_t kOffLen = align256(kOffCode + sizeof(uint32_t) * (kMaxKDPad / kMaxD) * kMaxDPad);   // (four qubits take the most)
+constexpr size_t kOffColw = align256(kOffLen + sizeof(uint16_t) * (kMaxKDPad / 8));
+static_assert(kOffColw + sizeof(float4) * kMaxKDPad / 2 <= kScratchBytes, "lists");
 static_assert(kScratchBytes == QST_NOALLOC_SCRATCH_BYTES, "qst.h states the scratch size");
 
 // The scratch itself.  In host code this name is only a host-side stand-in for the device
@@ -88,11 +96,15 @@ struct NoallocWeights {
 };
 
 __global__ void noalloc_weights_kernel(const __grid_constant__ NoallocWeights w, float *cnt, float *invf,
-                                       float *ptot) {
+                                       float *ptot, float4 *colw) {
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < w.n; m += gridDim.x * blockDim.x) {
         cnt[m] = w.cnt[m];
         invf[m] = w.invf[m];
         if (m < w.nk) ptot[m] = w.ptot[m];
+        if (colw && m % 2 == 0) {   // the pair's (invf, invf, add, add), as qst_create forms them
+            const bool c0 = w.cnt[m] > 0.0f, c1 = w.cnt[m + 1] > 0.0f;
+            colw[m / 2] = make_float4(c0 ? w.invf[m] : 0.0f, c1 ? w.invf[m + 1] : 0.0f, c0 ? 0.0f : 1.0f, c1 ? 0.0f : 1.0f);
+        }
     }
 }
 
@@ -171,15 +183,30 @@ extern "C" qst_status qst_loglik_noalloc(int32_t num_qubits, int32_t num_povms, 
     v.ngroups = fp32_ngroups(v, n);
 
     // The scratch keeps the previous call's contents: rewrite everything this call reads.
-    float *P32 = reinterpret_cast<float *>(scratch + kOffP);
-    cudaError_t e = cudaMemsetAsync(P32, 0, sizeof(float) * (size_t)d_pad * KD_pad, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpy2DAsync(P32, sizeof(float) * KD_pad, P, sizeof(float) * KD, sizeof(float) * KD, d,
-                              cudaMemcpyDeviceToDevice, s);
+    cudaError_t e = cudaSuccess;
+    float4 *colw = nullptr;
+    if (fp32_lists(v)) {
+        // three and four qubits: the lists of P's used rows, straight from the caller's matrix -- their
+        // values where the padded matrix would be, the rest behind at most kListGroups groups of partials
+        v.ngroups = std::min(v.ngroups, kListGroups);
+        v.sp_val = reinterpret_cast<const float *>(scratch + kOffP);
+        v.sp_code = reinterpret_cast<const uint32_t *>(scratch + kOffCode);
+        v.sp_len = reinterpret_cast<const uint16_t *>(scratch + kOffLen);
+        v.colw = colw = reinterpret_cast<float4 *>(scratch + kOffColw);
+        e = launch_fp32_lists(v, P, KD, reinterpret_cast<float *>(scratch + kOffP),
+                              reinterpret_cast<uint32_t *>(scratch + kOffCode),
+                              reinterpret_cast<uint16_t *>(scratch + kOffLen), s);
+    } else {
+        float *P32 = reinterpret_cast<float *>(scratch + kOffP);
+        e = cudaMemsetAsync(P32, 0, sizeof(float) * (size_t)d_pad * KD_pad, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpy2DAsync(P32, sizeof(float) * KD_pad, P, sizeof(float) * KD, sizeof(float) * KD, d,
+                                  cudaMemcpyDeviceToDevice, s);
+    }
     if (e == cudaSuccess) {
         noalloc_weights_kernel<<<(KD_pad + 255) / 256, 256, 0, s>>>(w, reinterpret_cast<float *>(scratch + kOffCnt),
                                                                    reinterpret_cast<float *>(scratch + kOffInvf),
-                                                                   reinterpret_cast<float *>(scratch + kOffPtot));
+                                                                   reinterpret_cast<float *>(scratch + kOffPtot), colw);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && d < d_pad)   // padding columns of the operand must be zero
