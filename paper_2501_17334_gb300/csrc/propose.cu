@@ -4,9 +4,13 @@
 // blocks G and H (the latent layout is column-major, so a column is D contiguous
 // floats of each of the four parts).  Per chain:
 //   1. eta from Philox (tag 1, step j) and y' = sqrt(1 - beta^2) y + beta eta, one
-//      Philox block (four entries) at a time; y' goes to the chain's other y buffer (the
-//      accept kernel flips to it); lane j keeps H's column j in registers.  G's column is
-//      read back from those same (own) global writes in step 3.
+//      Philox block (four entries) at a time, a chain's lanes on consecutive blocks; y' goes to the
+//      chain's other y buffer (the accept kernel flips to it); lane j takes H's column j through
+//      shared memory and keeps it in registers.  G's columns are read back from y' in step 3.
+//      (With every lane on its own column's blocks an access touched 32 pieces of 16 bytes in as
+//      many sectors or lines; consecutive blocks took the kernel from 536 to 524 us at 65536
+//      four-qubit chains, from 292 to 258 us at 8192 five-qubit ones and from 348 to 332 us at
+//      1024 six-qubit ones.)
 //   2. QR of H (Algorithm 1).  Modified Gram-Schmidt: at step k lane k publishes its
 //      (unnormalised) column v_k, and every lane j > k loads it, forms |v_k|^2 and v_k^dag h_j
 //      itself and removes the projection -- no lane works alone on a normalisation.  The
@@ -100,26 +104,37 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
     const uint32_t tag = (a.mode == MODE_INIT) ? TAG_INIT : TAG_PROPOSAL;
     const float *ysrc = a.y + ((int64_t)cur * a.R + cc) * nx;
     float *ydst = a.y + ((int64_t)(1 - cur) * a.R + cc) * nx;
-    // where G's column j is read back in step 3: this lane's own y' writes, or the input row
+    // where G's column j is read back in step 3: this chain's y' writes, or the input row
     const float *gsrc = (a.mode == MODE_EVAL) ? a.x_eval + cc * nx : ydst;
     float2 hr[D / 2], hi[D / 2];   // H's column j, entries (2p, 2p + 1) in pair p
     if constexpr (D >= 4) {
-        // lane j owns entries j D .. j D + D - 1 of each part: D/4 Philox blocks per part
+        // A part is d/4 Philox blocks of four entries.  Lane j takes blocks j, j + D, ..: a chain's
+        // lanes then read and write consecutive 16-byte pieces of y, and H's blocks reach the lanes that own
+        // their columns through shared memory (area B where the refinement keeps H's columns
+        // anyway, the Q planes otherwise).
+        constexpr int BPC = D / 4;   // blocks per column
+        auto stage = [&](float *plane_h, float *plane_q, int blk, float4 v) {
+            const int col = blk / BPC, r = blk % BPC;
+            if constexpr (PASSES == 3)
+                *reinterpret_cast<float4 *>(plane_h + col * D + 4 * (r ^ hsw<D, QC>(col))) = v;
+            else
+                *reinterpret_cast<float4 *>(plane_q + col * QC + 4 * (r ^ qsw<D, QC>(col))) = v;
+        };
 #pragma unroll 1
         for (int part = 0; part < 4; ++part) {
-            const int e0 = part * d + j * D;    // element index of (row 0, column j)
+            const int e0 = part * d + 4 * j;    // element index of this lane's first block
             float4 y0[D / 4];
 #pragma unroll
             for (int q = 0; q < D / 4; ++q) {
                 y0[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (active && a.mode == MODE_STEP) y0[q] = *reinterpret_cast<const float4 *>(ysrc + e0 + 4 * q);
-                if (active && a.mode == MODE_EVAL) y0[q] = *reinterpret_cast<const float4 *>(a.x_eval + cc * nx + e0 + 4 * q);
+                if (active && a.mode == MODE_STEP) y0[q] = *reinterpret_cast<const float4 *>(ysrc + e0 + 4 * D * q);
+                if (active && a.mode == MODE_EVAL) y0[q] = *reinterpret_cast<const float4 *>(a.x_eval + cc * nx + e0 + 4 * D * q);
             }
 #pragma unroll
             for (int q = 0; q < D / 4; ++q) {
                 float4 yn = y0[q];
                 if (a.mode != MODE_EVAL) {
-                    const uint4 w = Philox::block(make_uint4((uint32_t)(e0 / 4 + q), step, chain_id, tag), a.rk);
+                    const uint4 w = Philox::block(make_uint4((uint32_t)(e0 / 4 + D * q), step, chain_id, tag), a.rk);
                     float z0, z1, z2, z3;
                     gaussian_pair_fast(w.x, w.y, z0, z1);
                     gaussian_pair_fast(w.z, w.w, z2, z3);
@@ -127,16 +142,20 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
                     yn.y = __fmaf_rn(coef_y, y0[q].y, coef_eta * z1);
                     yn.z = __fmaf_rn(coef_y, y0[q].z, coef_eta * z2);
                     yn.w = __fmaf_rn(coef_y, y0[q].w, coef_eta * z3);
-                    if (active) *reinterpret_cast<float4 *>(ydst + e0 + 4 * q) = yn;
+                    if (active) *reinterpret_cast<float4 *>(ydst + e0 + 4 * D * q) = yn;
                 }
-                if (part == 2) {
-                    hr[2 * q] = make_float2(yn.x, yn.y);
-                    hr[2 * q + 1] = make_float2(yn.z, yn.w);
-                } else if (part == 3) {
-                    hi[2 * q] = make_float2(yn.x, yn.y);
-                    hi[2 * q + 1] = make_float2(yn.z, yn.w);
-                }
+                if (part == 2) stage(hre, qre, j + D * q, yn);
+                if (part == 3) stage(him, qim, j + D * q, yn);
             }
+        }
+        __syncwarp();
+        if constexpr (PASSES == 3) {
+            load_column2<D>(hre + j * D, hr, hsw<D, QC>(j));
+            load_column2<D>(him + j * D, hi, hsw<D, QC>(j));
+        } else {
+            load_column2<D>(qre + j * QC, hr, qsw<D, QC>(j));
+            load_column2<D>(qim + j * QC, hi, qsw<D, QC>(j));
+            __syncwarp();   // (the sweep publishes its columns there)
         }
     } else {
         // D == 2: each part is one Philox block shared by the two lanes; lane j takes pair j
@@ -173,7 +192,7 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
         }
     }
 
-    if constexpr (PASSES == 3) {   // H's original columns, for the refinement after the sweep
+    if constexpr (PASSES == 3 && D < 4) {   // H's original columns, for the refinement after the sweep (above for D >= 4)
         store_column2<D>(hre + j * D, hr, hsw<D, QC>(j));
         store_column2<D>(him + j * D, hi, hsw<D, QC>(j));
     }
@@ -564,6 +583,69 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
     }
 }
 
+// W = G + U G for one lane's block of 4 rows x 8 columns: rows 4 bi .. 4 bi + 3, columns 4 bj .. and
+// HALF + 4 bj ...  U column-major at stride qc (entry i of a column at at(i)), G row-major [D][D];
+// W's real and imaginary planes replace U's, row-major at stride qc (entry i of a row at at(i)),
+// after `sync` has seen every lane done with U.  An entry is sum_k U_ik G_kj in k's order (the two
+// products of a part one FMA after the other), then G_ij added.
+template <int D, int HALF, bool HAS_U, class At, class Sync>
+__device__ __forceinline__ void w_blocks(float *qre, float *qim, const float *gsr, const float *gsi, int bi, int bj, int qc,
+                                         At at, Sync sync) {
+    float2 wr[4][4], wi[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) wr[r][h] = wi[r][h] = make_float2(0.f, 0.f);
+    auto row_pairs = [&](const float *g, int row, float2 (&v)[4]) {
+        const float4 x = *reinterpret_cast<const float4 *>(g + row * D + 4 * bj);
+        const float4 y = *reinterpret_cast<const float4 *>(g + row * D + HALF + 4 * bj);
+        v[0] = make_float2(x.x, x.y);
+        v[1] = make_float2(x.z, x.w);
+        v[2] = make_float2(y.x, y.y);
+        v[3] = make_float2(y.z, y.w);
+    };
+    if constexpr (HAS_U) {
+#pragma unroll 2
+        for (int k = 0; k < D; ++k) {
+            const float4 ur4 = *reinterpret_cast<const float4 *>(qre + k * qc + at(4 * bi));
+            const float4 ui4 = *reinterpret_cast<const float4 *>(qim + k * qc + at(4 * bi));
+            float2 gr2[4], gi2[4];
+            row_pairs(gsr, k, gr2);
+            row_pairs(gsi, k, gi2);
+            const float ur[4] = {ur4.x, ur4.y, ur4.z, ur4.w}, ui[4] = {ui4.x, ui4.y, ui4.z, ui4.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float2 pu = make_float2(ur[r], ur[r]), pi = make_float2(ui[r], ui[r]);
+                const float2 mi = make_float2(-ui[r], -ui[r]);
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    wr[r][h] = __ffma2_rn(pu, gr2[h], __ffma2_rn(mi, gi2[h], wr[r][h]));
+                    wi[r][h] = __ffma2_rn(pu, gi2[h], __ffma2_rn(pi, gr2[h], wi[r][h]));
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        float2 g[4];
+        row_pairs(gsr, 4 * bi + r, g);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) wr[r][h] = __fadd2_rn(wr[r][h], g[h]);
+        row_pairs(gsi, 4 * bi + r, g);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) wi[r][h] = __fadd2_rn(wi[r][h], g[h]);
+    }
+    sync();   // U is read by every lane before W replaces it
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        float *re = qre + (4 * bi + r) * qc, *im = qim + (4 * bi + r) * qc;
+        *reinterpret_cast<float4 *>(re + at(4 * bj)) = make_float4(wr[r][0].x, wr[r][0].y, wr[r][1].x, wr[r][1].y);
+        *reinterpret_cast<float4 *>(re + at(HALF + 4 * bj)) = make_float4(wr[r][2].x, wr[r][2].y, wr[r][3].x, wr[r][3].y);
+        *reinterpret_cast<float4 *>(im + at(4 * bj)) = make_float4(wi[r][0].x, wi[r][0].y, wi[r][1].x, wi[r][1].y);
+        *reinterpret_cast<float4 *>(im + at(HALF + 4 * bj)) = make_float4(wi[r][2].x, wi[r][2].y, wi[r][3].x, wi[r][3].y);
+    }
+}
+
 // ---- five qubits (D = 32): one warp per chain ----------------------------------------------
 // The same algorithm with the same lane ownership (lane j: column j, then row j), but at D = 32 a
 // lane cannot also hold the operand it is multiplied with, so that operand is streamed from
@@ -604,7 +686,8 @@ __global__ void __launch_bounds__(THREADS, 3 * kThreads / THREADS) propose_kerne
     float *hre = sm + S::area_a, *him = hre + D * D;     // PASSES = 3: H's columns (stride D), in area B
     float2 *rpk = reinterpret_cast<float2 *>(sm + S::area_a + S::area_b);   // PASSES = 3: packed R
 
-    // ---- 1. latent proposal (as in the D <= 16 kernel: lane j owns column j of each part) ------
+    // ---- 1. latent proposal (as in the D <= 16 kernel: lane j takes blocks j, j + 32, .. of each part,
+    // H's blocks go through the Q planes to the lanes that own their columns) ---------------------
     float coef_y = 1.0f, coef_eta = 0.0f;
     int cur = 0;
     if (active && a.mode == MODE_STEP) {
@@ -625,33 +708,37 @@ __global__ void __launch_bounds__(THREADS, 3 * kThreads / THREADS) propose_kerne
     float2 hr[D / 2], hi[D / 2];   // H's column j, entries (2p, 2p + 1) in pair p
 #pragma unroll 1
     for (int part = 0; part < 4; ++part) {
-        const int e0 = part * d + j * D;
+        const int e0 = part * d + 4 * j;
+        float4 y0[D / 4];
 #pragma unroll
         for (int q = 0; q < D / 4; ++q) {
-            float4 y0 = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (active && a.mode == MODE_STEP) y0 = *reinterpret_cast<const float4 *>(ysrc + e0 + 4 * q);
-            if (active && a.mode == MODE_EVAL) y0 = *reinterpret_cast<const float4 *>(a.x_eval + cc * nx + e0 + 4 * q);
-            float4 yn = y0;
+            y0[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (active && a.mode == MODE_STEP) y0[q] = *reinterpret_cast<const float4 *>(ysrc + e0 + 4 * D * q);
+            if (active && a.mode == MODE_EVAL) y0[q] = *reinterpret_cast<const float4 *>(a.x_eval + cc * nx + e0 + 4 * D * q);
+        }
+#pragma unroll
+        for (int q = 0; q < D / 4; ++q) {
+            float4 yn = y0[q];
             if (a.mode != MODE_EVAL) {
-                const uint4 w = Philox::block(make_uint4((uint32_t)(e0 / 4 + q), step, chain_id, tag), a.rk);
+                const uint4 w = Philox::block(make_uint4((uint32_t)(e0 / 4 + D * q), step, chain_id, tag), a.rk);
                 float z0, z1, z2, z3;
                 gaussian_pair_fast(w.x, w.y, z0, z1);
                 gaussian_pair_fast(w.z, w.w, z2, z3);
-                yn.x = __fmaf_rn(coef_y, y0.x, coef_eta * z0);
-                yn.y = __fmaf_rn(coef_y, y0.y, coef_eta * z1);
-                yn.z = __fmaf_rn(coef_y, y0.z, coef_eta * z2);
-                yn.w = __fmaf_rn(coef_y, y0.w, coef_eta * z3);
-                if (active) *reinterpret_cast<float4 *>(ydst + e0 + 4 * q) = yn;
+                yn.x = __fmaf_rn(coef_y, y0[q].x, coef_eta * z0);
+                yn.y = __fmaf_rn(coef_y, y0[q].y, coef_eta * z1);
+                yn.z = __fmaf_rn(coef_y, y0[q].z, coef_eta * z2);
+                yn.w = __fmaf_rn(coef_y, y0[q].w, coef_eta * z3);
+                if (active) *reinterpret_cast<float4 *>(ydst + e0 + 4 * D * q) = yn;
             }
-            if (part == 2) {
-                hr[2 * q] = make_float2(yn.x, yn.y);
-                hr[2 * q + 1] = make_float2(yn.z, yn.w);
-            } else if (part == 3) {
-                hi[2 * q] = make_float2(yn.x, yn.y);
-                hi[2 * q + 1] = make_float2(yn.z, yn.w);
-            }
+            const int blk = j + D * q, at = blk / (D / 4) * QC + 4 * (blk % (D / 4));
+            if (part == 2) *reinterpret_cast<float4 *>(qre + at) = yn;
+            if (part == 3) *reinterpret_cast<float4 *>(qim + at) = yn;
         }
     }
+    __syncwarp();
+    load_column2<D>(qre + j * QC, hr);
+    load_column2<D>(qim + j * QC, hi);
+    __syncwarp();   // (the sweep publishes its columns there)
     if constexpr (PASSES == 3) {   // H's original columns, for the refinement after the sweep
         store_column2<D>(hre + j * D, hr);
         store_column2<D>(him + j * D, hi);
@@ -669,22 +756,20 @@ __global__ void __launch_bounds__(THREADS, 3 * kThreads / THREADS) propose_kerne
             store_column2<D>(qim + k * QC, hi);
         }
         __syncwarp();
-        const float *vre = qre + k * QC, *vim = qim + k * QC;
+        float2 vr[D / 2], vi[D / 2];   // held for the projection too: the broadcast loads are what bounds the sweep
+        load_column2<D>(qre + k * QC, vr);
+        load_column2<D>(qim + k * QC, vi);
         float2 a0 = make_float2(0.f, 0.f), a1 = a0, a2 = a0, a3 = a0, b0 = a0, b1 = a0, b2 = a0, b3 = a0;
 #pragma unroll
         for (int p = 0; p < D / 2; p += 2) {
-            const float4 vr4 = *reinterpret_cast<const float4 *>(vre + 2 * p);
-            const float4 vi4 = *reinterpret_cast<const float4 *>(vim + 2 * p);
-            const float2 vr0 = make_float2(vr4.x, vr4.y), vr1 = make_float2(vr4.z, vr4.w);
-            const float2 vi0 = make_float2(vi4.x, vi4.y), vi1 = make_float2(vi4.z, vi4.w);
-            a0 = __ffma2_rn(vr0, hr[p], a0);
-            a1 = __ffma2_rn(vi0, hi[p], a1);
-            b0 = __ffma2_rn(vr0, hi[p], b0);
-            b1 = __ffma2_rn(vi0, hr[p], b1);
-            a2 = __ffma2_rn(vr1, hr[p + 1], a2);
-            a3 = __ffma2_rn(vi1, hi[p + 1], a3);
-            b2 = __ffma2_rn(vr1, hi[p + 1], b2);
-            b3 = __ffma2_rn(vi1, hr[p + 1], b3);
+            a0 = __ffma2_rn(vr[p], hr[p], a0);
+            a1 = __ffma2_rn(vi[p], hi[p], a1);
+            b0 = __ffma2_rn(vr[p], hi[p], b0);
+            b1 = __ffma2_rn(vi[p], hr[p], b1);
+            a2 = __ffma2_rn(vr[p + 1], hr[p + 1], a2);
+            a3 = __ffma2_rn(vi[p + 1], hi[p + 1], a3);
+            b2 = __ffma2_rn(vr[p + 1], hi[p + 1], b2);
+            b3 = __ffma2_rn(vi[p + 1], hr[p + 1], b3);
         }
         const float rr = (hsum(a0) + hsum(a1)) + (hsum(a2) + hsum(a3));
         const float ri = (hsum(b0) - hsum(b1)) + (hsum(b2) - hsum(b3));
@@ -694,15 +779,9 @@ __global__ void __launch_bounds__(THREADS, 3 * kThreads / THREADS) propose_kerne
         const float sr = rr * coef, si = ri * coef;
         const float2 msr = make_float2(-sr, -sr), psi = make_float2(si, si), msi = make_float2(-si, -si);
 #pragma unroll
-        for (int p = 0; p < D / 2; p += 2) {
-            const float4 vr4 = *reinterpret_cast<const float4 *>(vre + 2 * p);
-            const float4 vi4 = *reinterpret_cast<const float4 *>(vim + 2 * p);
-            const float2 vr0 = make_float2(vr4.x, vr4.y), vr1 = make_float2(vr4.z, vr4.w);
-            const float2 vi0 = make_float2(vi4.x, vi4.y), vi1 = make_float2(vi4.z, vi4.w);
-            hr[p] = __ffma2_rn(msr, vr0, __ffma2_rn(psi, vi0, hr[p]));
-            hi[p] = __ffma2_rn(msr, vi0, __ffma2_rn(msi, vr0, hi[p]));
-            hr[p + 1] = __ffma2_rn(msr, vr1, __ffma2_rn(psi, vi1, hr[p + 1]));
-            hi[p + 1] = __ffma2_rn(msr, vi1, __ffma2_rn(msi, vr1, hi[p + 1]));
+        for (int p = 0; p < D / 2; ++p) {
+            hr[p] = __ffma2_rn(msr, vr[p], __ffma2_rn(psi, vi[p], hr[p]));
+            hi[p] = __ffma2_rn(msr, vi[p], __ffma2_rn(msi, vr[p], hi[p]));
         }
         inv_own = (j == k) ? rs : inv_own;
         if constexpr (PASSES == 2) {
@@ -799,62 +878,33 @@ __global__ void __launch_bounds__(THREADS, 3 * kThreads / THREADS) propose_kerne
         __syncwarp();
     }
 
-    // ---- 3. W[:, j] = G[:, j] + sum_k U[:, k] G[k, j]: pairs of rows, U streamed, G[k, j] broadcast
-    float2 wr[D / 2], wi[D / 2];
+    // ---- 3. W = G + U G in blocks of 4 rows x 8 columns per lane (rows 4 bi .., columns 4 bj .. and
+    // 16 + 4 bj ..), each entry the sum over k in order and then G's entry: a k costs six 128-bit
+    // loads, of which a warp reads 128 bytes each at most, where column j per lane took sixteen
+    // broadcast ones.  G is staged row-major as real and imaginary planes in area B.
+    {
+        float *gsr = sm + S::area_a, *gsi = gsr + D * D;
 #pragma unroll
-    for (int p = 0; p < D / 2; ++p) wr[p] = wi[p] = make_float2(0.f, 0.f);
-    // G[k0..k0+3, j] from y' (L2), requested one group ahead of its use
-    float4 g4r_next = make_float4(0.f, 0.f, 0.f, 0.f), g4i_next = g4r_next;
-    if (active && PASSES > 0) {
-        g4r_next = *reinterpret_cast<const float4 *>(gsrc + j * D);
-        g4i_next = *reinterpret_cast<const float4 *>(gsrc + d + j * D);
-    }
-#pragma unroll 1
-    for (int k0 = 0; k0 < (PASSES > 0 ? D : 0); k0 += 4) {
-        const float4 g4r = g4r_next, g4i = g4i_next;
-        if (active && k0 + 4 < D) {
-            g4r_next = *reinterpret_cast<const float4 *>(gsrc + j * D + k0 + 4);
-            g4i_next = *reinterpret_cast<const float4 *>(gsrc + d + j * D + k0 + 4);
-        }
-        const float gkr[4] = {g4r.x, g4r.y, g4r.z, g4r.w}, gki[4] = {g4i.x, g4i.y, g4i.z, g4i.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const float *ure = qre + (k0 + u) * QC, *uim = qim + (k0 + u) * QC;
-            const float2 pgr = make_float2(gkr[u], gkr[u]), pgi = make_float2(gki[u], gki[u]);
-            const float2 mgi = make_float2(-gki[u], -gki[u]);
-#pragma unroll
-            for (int p = 0; p < D / 2; p += 2) {
-                const float4 ur = *reinterpret_cast<const float4 *>(ure + 2 * p);
-                const float4 ui = *reinterpret_cast<const float4 *>(uim + 2 * p);
-                const float2 ur0 = make_float2(ur.x, ur.y), ur1 = make_float2(ur.z, ur.w);
-                const float2 ui0 = make_float2(ui.x, ui.y), ui1 = make_float2(ui.z, ui.w);
-                wr[p] = __ffma2_rn(ur0, pgr, __ffma2_rn(ui0, mgi, wr[p]));
-                wi[p] = __ffma2_rn(ur0, pgi, __ffma2_rn(ui0, pgr, wi[p]));
-                wr[p + 1] = __ffma2_rn(ur1, pgr, __ffma2_rn(ui1, mgi, wr[p + 1]));
-                wi[p + 1] = __ffma2_rn(ur1, pgi, __ffma2_rn(ui1, pgr, wi[p + 1]));
+        for (int q = 0; q < D / 4; ++q) {
+            float4 g4r = make_float4(0.f, 0.f, 0.f, 0.f), g4i = g4r;
+            if (active) {
+                g4r = *reinterpret_cast<const float4 *>(gsrc + j * D + 4 * q);
+                g4i = *reinterpret_cast<const float4 *>(gsrc + d + j * D + 4 * q);
             }
+            gsr[(4 * q) * D + j] = g4r.x;
+            gsr[(4 * q + 1) * D + j] = g4r.y;
+            gsr[(4 * q + 2) * D + j] = g4r.z;
+            gsr[(4 * q + 3) * D + j] = g4r.w;
+            gsi[(4 * q) * D + j] = g4i.x;
+            gsi[(4 * q + 1) * D + j] = g4i.y;
+            gsi[(4 * q + 2) * D + j] = g4i.z;
+            gsi[(4 * q + 3) * D + j] = g4i.w;
         }
+        __syncwarp();
+        w_blocks<D, 16, (PASSES > 0)>(qre, qim, gsr, gsi, j >> 2, j & 3, QC, [](int i) { return i; },
+                                            [] { __syncwarp(); });
+        __syncwarp();
     }
-    if (active) {   // + G[:, j]
-#pragma unroll
-        for (int p = 0; p < D / 2; p += 2) {
-            const float4 gr4 = *reinterpret_cast<const float4 *>(gsrc + j * D + 2 * p);
-            const float4 gi4 = *reinterpret_cast<const float4 *>(gsrc + d + j * D + 2 * p);
-            wr[p] = __fadd2_rn(wr[p], make_float2(gr4.x, gr4.y));
-            wr[p + 1] = __fadd2_rn(wr[p + 1], make_float2(gr4.z, gr4.w));
-            wi[p] = __fadd2_rn(wi[p], make_float2(gi4.x, gi4.y));
-            wi[p + 1] = __fadd2_rn(wi[p + 1], make_float2(gi4.z, gi4.w));
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int p = 0; p < D / 2; ++p) {   // W row-major, real and imaginary planes (replace Q)
-        wre[(2 * p) * QC + j] = wr[p].x;
-        wre[(2 * p + 1) * QC + j] = wr[p].y;
-        wim[(2 * p) * QC + j] = wi[p].x;
-        wim[(2 * p + 1) * QC + j] = wi[p].y;
-    }
-    __syncwarp();
 
     // ---- 4. rho = W W^dag / Tr, lane a: entries (a, a + t mod D), row b streamed --------------
     // Re (W W^dag)_ab = sum Re W_am Re W_bm + Im W_am Im W_bm and Im = sum Im W_am Re W_bm -
@@ -1004,34 +1054,39 @@ __global__ void __launch_bounds__(Wide64::threads, 3) propose_kernel_d64(Propose
     float2 hr[H2 / 2], hi[H2 / 2];   // rows r0 + 2p, r0 + 2p + 1 of H's column j in pair p
 #pragma unroll 1
     for (int part = 0; part < 4; ++part) {
-        const int e0 = part * d + j * D + r0;
+        // thread t takes blocks t, t + 128, ..; H's reach the threads that own them through the Q planes
+        const int e0 = part * d + 4 * t;
+        float4 y0[H2 / 4];
 #pragma unroll
         for (int q = 0; q < H2 / 4; ++q) {
-            float4 y0 = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (a.mode == MODE_STEP) y0 = *reinterpret_cast<const float4 *>(ysrc + e0 + 4 * q);
-            if (a.mode == MODE_EVAL) y0 = *reinterpret_cast<const float4 *>(a.x_eval + c * nx + e0 + 4 * q);
-            float4 yn = y0;
+            y0[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (a.mode == MODE_STEP) y0[q] = *reinterpret_cast<const float4 *>(ysrc + e0 + 4 * S::threads * q);
+            if (a.mode == MODE_EVAL) y0[q] = *reinterpret_cast<const float4 *>(a.x_eval + c * nx + e0 + 4 * S::threads * q);
+        }
+#pragma unroll
+        for (int q = 0; q < H2 / 4; ++q) {
+            float4 yn = y0[q];
             if (a.mode != MODE_EVAL) {
-                const uint4 w = Philox::block(make_uint4((uint32_t)(e0 / 4 + q), step, chain_id, tag), a.rk);
+                const uint4 w = Philox::block(make_uint4((uint32_t)(e0 / 4 + S::threads * q), step, chain_id, tag), a.rk);
                 float z0, z1, z2, z3;
                 gaussian_pair_fast(w.x, w.y, z0, z1);
                 gaussian_pair_fast(w.z, w.w, z2, z3);
-                yn.x = __fmaf_rn(coef_y, y0.x, coef_eta * z0);
-                yn.y = __fmaf_rn(coef_y, y0.y, coef_eta * z1);
-                yn.z = __fmaf_rn(coef_y, y0.z, coef_eta * z2);
-                yn.w = __fmaf_rn(coef_y, y0.w, coef_eta * z3);
-                *reinterpret_cast<float4 *>(ydst + e0 + 4 * q) = yn;
+                yn.x = __fmaf_rn(coef_y, y0[q].x, coef_eta * z0);
+                yn.y = __fmaf_rn(coef_y, y0[q].y, coef_eta * z1);
+                yn.z = __fmaf_rn(coef_y, y0[q].z, coef_eta * z2);
+                yn.w = __fmaf_rn(coef_y, y0[q].w, coef_eta * z3);
+                *reinterpret_cast<float4 *>(ydst + e0 + 4 * S::threads * q) = yn;
             }
-            if (part == 2) {
-                hr[2 * q] = make_float2(yn.x, yn.y);
-                hr[2 * q + 1] = make_float2(yn.z, yn.w);
-            } else if (part == 3) {
-                hi[2 * q] = make_float2(yn.x, yn.y);
-                hi[2 * q + 1] = make_float2(yn.z, yn.w);
-            }
+            const int blk = t + S::threads * q, r = blk % (D / 4);
+            const int at = blk / (D / 4) * QC + 4 * r + 4 * (r / (D / 8));
+            if (part == 2) *reinterpret_cast<float4 *>(qre + at) = yn;
+            if (part == 3) *reinterpret_cast<float4 *>(qim + at) = yn;
         }
     }
-    __syncthreads();   // y' (read back as G) is written
+    __syncthreads();   // y' (read back as G) is written, H staged
+    load_column2<H2>(qre + j * QC + r0s, hr);
+    load_column2<H2>(qim + j * QC + r0s, hi);
+    __syncthreads();   // (the sweep publishes its columns there)
 
     // ---- 2a. modified Gram-Schmidt: q_k = v_k / |v_k| published by its pair, projected out ------
 #pragma unroll 1
@@ -1053,18 +1108,16 @@ __global__ void __launch_bounds__(Wide64::threads, 3) propose_kernel_d64(Propose
         }
         __syncthreads();
         // r = q_k^dag h over this half, then both halves
-        const float *vre = qre + k * QC + r0s, *vim = qim + k * QC + r0s;
+        float2 vr[H2 / 2], vi[H2 / 2];   // held for the projection too
+        load_column2<H2>(qre + k * QC + r0s, vr);
+        load_column2<H2>(qim + k * QC + r0s, vi);
         float2 a0 = make_float2(0.f, 0.f), a1 = a0, b0 = a0, b1 = a0;
 #pragma unroll
         for (int p = 0; p < H2 / 2; p += 2) {
-            const float4 vr4 = *reinterpret_cast<const float4 *>(vre + 2 * p);
-            const float4 vi4 = *reinterpret_cast<const float4 *>(vim + 2 * p);
-            const float2 vr0 = make_float2(vr4.x, vr4.y), vr1 = make_float2(vr4.z, vr4.w);
-            const float2 vi0 = make_float2(vi4.x, vi4.y), vi1 = make_float2(vi4.z, vi4.w);
-            a0 = __ffma2_rn(vr0, hr[p], __ffma2_rn(vr1, hr[p + 1], a0));
-            a1 = __ffma2_rn(vi0, hi[p], __ffma2_rn(vi1, hi[p + 1], a1));
-            b0 = __ffma2_rn(vr0, hi[p], __ffma2_rn(vr1, hi[p + 1], b0));
-            b1 = __ffma2_rn(vi0, hr[p], __ffma2_rn(vi1, hr[p + 1], b1));
+            a0 = __ffma2_rn(vr[p], hr[p], __ffma2_rn(vr[p + 1], hr[p + 1], a0));
+            a1 = __ffma2_rn(vi[p], hi[p], __ffma2_rn(vi[p + 1], hi[p + 1], a1));
+            b0 = __ffma2_rn(vr[p], hi[p], __ffma2_rn(vr[p + 1], hi[p + 1], b0));
+            b1 = __ffma2_rn(vi[p], hr[p], __ffma2_rn(vi[p + 1], hr[p + 1], b1));
         }
         float rr = hsum(a0) + hsum(a1), ri = hsum(b0) - hsum(b1);
         rr += __shfl_xor_sync(0xffffffffu, rr, 1);
@@ -1072,15 +1125,9 @@ __global__ void __launch_bounds__(Wide64::threads, 3) propose_kernel_d64(Propose
         if (j > k) {   // h -= r q_k
             const float2 msr = make_float2(-rr, -rr), psi = make_float2(ri, ri), msi = make_float2(-ri, -ri);
 #pragma unroll
-            for (int p = 0; p < H2 / 2; p += 2) {
-                const float4 vr4 = *reinterpret_cast<const float4 *>(vre + 2 * p);
-                const float4 vi4 = *reinterpret_cast<const float4 *>(vim + 2 * p);
-                const float2 vr0 = make_float2(vr4.x, vr4.y), vr1 = make_float2(vr4.z, vr4.w);
-                const float2 vi0 = make_float2(vi4.x, vi4.y), vi1 = make_float2(vi4.z, vi4.w);
-                hr[p] = __ffma2_rn(msr, vr0, __ffma2_rn(psi, vi0, hr[p]));
-                hi[p] = __ffma2_rn(msr, vi0, __ffma2_rn(msi, vr0, hi[p]));
-                hr[p + 1] = __ffma2_rn(msr, vr1, __ffma2_rn(psi, vi1, hr[p + 1]));
-                hi[p + 1] = __ffma2_rn(msr, vi1, __ffma2_rn(msi, vr1, hi[p + 1]));
+            for (int p = 0; p < H2 / 2; ++p) {
+                hr[p] = __ffma2_rn(msr, vr[p], __ffma2_rn(psi, vi[p], hr[p]));
+                hi[p] = __ffma2_rn(msr, vi[p], __ffma2_rn(msi, vr[p], hi[p]));
             }
         } else if (PASSES == 2 && j < k && hh == 0) {   // E_jk = q_j^dag q_k = conj(q_k^dag q_j)
             fre[k * D + j] = rr;
@@ -1126,51 +1173,26 @@ __global__ void __launch_bounds__(Wide64::threads, 3) propose_kernel_d64(Propose
         __syncthreads();
     }
 
-    // ---- 3. W[:, j] = G[:, j] + sum_k U[:, k] G[k, j] over this half's rows --------------------
-    float2 wr[H2 / 2], wi[H2 / 2];
+    // ---- 3. W = G + U G in blocks of 4 rows x 8 columns per thread (w_blocks), G staged row-major in
+    // area B (F is no longer needed) ------------------------------------------------------------------
+    {
+        float *gsr = smem + S::area_a, *gsi = gsr + D * D;
 #pragma unroll
-    for (int p = 0; p < H2 / 2; ++p) wr[p] = wi[p] = make_float2(0.f, 0.f);
-#pragma unroll 1
-    for (int k0 = 0; k0 < (PASSES > 0 ? D : 0); k0 += 4) {
-        const float4 g4r = *reinterpret_cast<const float4 *>(gsrc + j * D + k0);
-        const float4 g4i = *reinterpret_cast<const float4 *>(gsrc + d + j * D + k0);
-        const float gkr[4] = {g4r.x, g4r.y, g4r.z, g4r.w}, gki[4] = {g4i.x, g4i.y, g4i.z, g4i.w};
+        for (int q = 0; q < H2 / 4; ++q) {
+            const float4 g4r = *reinterpret_cast<const float4 *>(gsrc + j * D + r0 + 4 * q);
+            const float4 g4i = *reinterpret_cast<const float4 *>(gsrc + d + j * D + r0 + 4 * q);
+            const float gr[4] = {g4r.x, g4r.y, g4r.z, g4r.w}, gi[4] = {g4i.x, g4i.y, g4i.z, g4i.w};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const float *ure = qre + (k0 + u) * QC + r0s, *uim = qim + (k0 + u) * QC + r0s;
-            const float2 pgr = make_float2(gkr[u], gkr[u]), pgi = make_float2(gki[u], gki[u]);
-            const float2 mgi = make_float2(-gki[u], -gki[u]);
-#pragma unroll
-            for (int p = 0; p < H2 / 2; p += 2) {
-                const float4 ur = *reinterpret_cast<const float4 *>(ure + 2 * p);
-                const float4 ui = *reinterpret_cast<const float4 *>(uim + 2 * p);
-                const float2 ur0 = make_float2(ur.x, ur.y), ur1 = make_float2(ur.z, ur.w);
-                const float2 ui0 = make_float2(ui.x, ui.y), ui1 = make_float2(ui.z, ui.w);
-                wr[p] = __ffma2_rn(ur0, pgr, __ffma2_rn(ui0, mgi, wr[p]));
-                wi[p] = __ffma2_rn(ur0, pgi, __ffma2_rn(ui0, pgr, wi[p]));
-                wr[p + 1] = __ffma2_rn(ur1, pgr, __ffma2_rn(ui1, mgi, wr[p + 1]));
-                wi[p + 1] = __ffma2_rn(ur1, pgi, __ffma2_rn(ui1, pgr, wi[p + 1]));
+            for (int u = 0; u < 4; ++u) {
+                gsr[(r0 + 4 * q + u) * D + j] = gr[u];
+                gsi[(r0 + 4 * q + u) * D + j] = gi[u];
             }
         }
+        __syncthreads();
+        w_blocks<D, H2, (PASSES > 0)>(qre, qim, gsr, gsi, t >> 3, t & 7, QC, [](int i) { return i + 4 * (i >> 5); },
+                                      [] { __syncthreads(); });
+        __syncthreads();
     }
-#pragma unroll
-    for (int p = 0; p < H2 / 2; p += 2) {   // + G[:, j]
-        const float4 gr4 = *reinterpret_cast<const float4 *>(gsrc + j * D + r0 + 2 * p);
-        const float4 gi4 = *reinterpret_cast<const float4 *>(gsrc + d + j * D + r0 + 2 * p);
-        wr[p] = __fadd2_rn(wr[p], make_float2(gr4.x, gr4.y));
-        wr[p + 1] = __fadd2_rn(wr[p + 1], make_float2(gr4.z, gr4.w));
-        wi[p] = __fadd2_rn(wi[p], make_float2(gi4.x, gi4.y));
-        wi[p + 1] = __fadd2_rn(wi[p + 1], make_float2(gi4.z, gi4.w));
-    }
-    __syncthreads();   // U is read by every thread before W replaces it
-#pragma unroll
-    for (int p = 0; p < H2 / 2; ++p) {   // W row-major, real and imaginary planes
-        wre[(r0 + 2 * p) * QC + js] = wr[p].x;
-        wre[(r0 + 2 * p + 1) * QC + js] = wr[p].y;
-        wim[(r0 + 2 * p) * QC + js] = wi[p].x;
-        wim[(r0 + 2 * p + 1) * QC + js] = wi[p].y;
-    }
-    __syncthreads();
 
     // ---- 4. rho = W W^dag / Tr: row a = j, this thread's half of the columns m ------------------
     const int arow = j;
