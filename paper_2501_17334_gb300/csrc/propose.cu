@@ -1011,7 +1011,10 @@ struct Wide64 {
     static constexpr int qcol = D + 8;
     static constexpr int pk_stride = D + 1;
     static constexpr int area_a = 2 * D * qcol;         // Q planes, then W as two planes of row stride qcol
-    static constexpr int area_b = 2 * D * D;            // F planes (column-major), then the staged rho
+    // F's planes are row-major; 68 floats a row keep the sweep's stores (one row per column pair) to two
+    // rows per bank and the rows 16-byte aligned
+    static constexpr int frow = D + 4;
+    static constexpr int area_b = 2 * D * frow;         // F planes, then G's planes, then the staged rho
     static constexpr int smem_floats = area_a + area_b + 2 * D + 32;
 };
 static_assert(Wide64::area_b >= Wide64::D * Wide64::pk_stride, "areas");
@@ -1023,7 +1026,7 @@ __global__ void __launch_bounds__(Wide64::threads, 3) propose_kernel_d64(Propose
     extern __shared__ __align__(16) float smem[];
     float *qre = smem, *qim = smem + D * QC;             // Q planes (column stride QC)
     float *wre = smem, *wim = smem + D * QC;             // W planes (row stride QC), replace Q
-    float *fre = smem + S::area_a, *fim = fre + D * D;   // F column-major (F[p][m] at m D + p)
+    float *fre = smem + S::area_a, *fim = fre + D * S::frow;   // F row-major (F[p][m] at p frow + m)
     float *packed = smem + S::area_a;                    // staged rho (row stride PK), replaces F
     float *rowv = smem + S::area_a + S::area_b;          // [D] per-row values (diagonal of W W^dag)
     const int t = threadIdx.x;
@@ -1083,6 +1086,10 @@ __global__ void __launch_bounds__(Wide64::threads, 3) propose_kernel_d64(Propose
             if (part == 3) *reinterpret_cast<float4 *>(qim + at) = yn;
         }
     }
+    if constexpr (PASSES == 2) {   // F's entries below the diagonal count as zero
+        for (int e = 4 * t; e < 2 * D * S::frow; e += 4 * S::threads)
+            *reinterpret_cast<float4 *>(fre + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     __syncthreads();   // y' (read back as G) is written, H staged
     load_column2<H2>(qre + j * QC + r0s, hr);
     load_column2<H2>(qim + j * QC + r0s, hi);
@@ -1130,8 +1137,8 @@ __global__ void __launch_bounds__(Wide64::threads, 3) propose_kernel_d64(Propose
                 hi[p] = __ffma2_rn(msr, vi[p], __ffma2_rn(msi, vr[p], hi[p]));
             }
         } else if (PASSES == 2 && j < k && hh == 0) {   // E_jk = q_j^dag q_k = conj(q_k^dag q_j)
-            fre[k * D + j] = rr;
-            fim[k * D + j] = -ri;
+            fre[j * S::frow + k] = rr;
+            fim[j * S::frow + k] = -ri;
         }
     }
 
@@ -1143,31 +1150,81 @@ __global__ void __launch_bounds__(Wide64::threads, 3) propose_kernel_d64(Propose
             float n = hsum(n2);
             n += __shfl_xor_sync(0xffffffffu, n, 1);
             if (hh == 0) {
-                fre[j * D + j] = 0.5f * (n - 1.0f);
-                fim[j * D + j] = 0.0f;
+                fre[j * S::frow + j] = 0.5f * (n - 1.0f);
+                fim[j * S::frow + j] = 0.0f;
             }
         }
         __syncthreads();
-        // ---- 2b. Q2 = Q1 (I - F): row a = j, the columns m of parity hh ------------------------
-        float2 q2[H2];   // (re, im) of Q2[a][2 mm + hh]
-#pragma unroll 1
-        for (int mm = 0; mm < H2; ++mm) {
-            const int m = 2 * mm + hh;
-            float2 acc = make_float2(0.f, 0.f), acc2 = acc;   // sum_p Q1[a][p] F[p][m] as (re, im) pairs
-            for (int p = 0; p <= m; ++p) {
-                const float xr = qre[p * QC + js], xi = qim[p * QC + js];
-                const float fr = fre[m * D + p], fi = fim[m * D + p];
-                acc = __ffma2_rn(make_float2(xr, xr), make_float2(fr, fi), acc);     // (xr fr, xr fi)
-                acc2 = __ffma2_rn(make_float2(xi, xi), make_float2(fi, fr), acc2);   // (xi fi, xi fr)
-            }
-            q2[mm] = make_float2(qre[m * QC + js] - (acc.x - acc2.x), qim[m * QC + js] - (acc.y + acc2.y));
-        }
-        __syncthreads();
+        // ---- 2b. Q2 = Q1 (I - F) in blocks of 4 rows x 4 columns per thread: columns 32 .. 63 first (they
+        // need every column of Q1), then 0 .. 31 (which need those only).  An entry is Q1_am - sum over
+        // p of Q1_ap F_pm in p's order; the terms p > m of a block are zeros of F.  Warp w takes columns
+        // 8 w .. 8 w + 7 of the low half and the mirrored ones of the high half, so the warps' sums are
+        // equally long (72 terms).  (A row per thread pair, one column after the other, took four scalar
+        // loads for two packed FMAs: 332 us for 1024 chains, 263 this way.)
+        const int bi = t & 15, bj = t >> 4;
+        const int x0 = 4 * bi + 4 * (bi >> 3);   // where rows 4 bi .. sit within a column
+        float2 q2r[4][2], q2i[4][2];             // Q2 of the block, pairs of columns
+        auto block = [&](int m0, int terms) {    // columns m0 .. m0 + 3
+            float2 rr[4][2], ii[4][2], ri[4][2], ir[4][2];   // sums of xr fr, xi fi, xr fi, xi fr
 #pragma unroll
-        for (int mm = 0; mm < H2; ++mm) {
-            qre[(2 * mm + hh) * QC + js] = q2[mm].x;
-            qim[(2 * mm + hh) * QC + js] = q2[mm].y;
-        }
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int h2 = 0; h2 < 2; ++h2) rr[r][h2] = ii[r][h2] = ri[r][h2] = ir[r][h2] = make_float2(0.f, 0.f);
+#pragma unroll 2
+            for (int p = 0; p < terms; ++p) {
+                const float4 xr4 = *reinterpret_cast<const float4 *>(qre + p * QC + x0);
+                const float4 xi4 = *reinterpret_cast<const float4 *>(qim + p * QC + x0);
+                const float4 fr4 = *reinterpret_cast<const float4 *>(fre + p * S::frow + m0);
+                const float4 fi4 = *reinterpret_cast<const float4 *>(fim + p * S::frow + m0);
+                const float xr[4] = {xr4.x, xr4.y, xr4.z, xr4.w}, xi[4] = {xi4.x, xi4.y, xi4.z, xi4.w};
+                const float2 fr[2] = {make_float2(fr4.x, fr4.y), make_float2(fr4.z, fr4.w)};
+                const float2 fi[2] = {make_float2(fi4.x, fi4.y), make_float2(fi4.z, fi4.w)};
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float2 pr = make_float2(xr[r], xr[r]), pi = make_float2(xi[r], xi[r]);
+#pragma unroll
+                    for (int h2 = 0; h2 < 2; ++h2) {
+                        rr[r][h2] = __ffma2_rn(pr, fr[h2], rr[r][h2]);
+                        ii[r][h2] = __ffma2_rn(pi, fi[h2], ii[r][h2]);
+                        ri[r][h2] = __ffma2_rn(pr, fi[h2], ri[r][h2]);
+                        ir[r][h2] = __ffma2_rn(pi, fr[h2], ir[r][h2]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int c4 = 0; c4 < 4; ++c4) {
+                const float4 xr4 = *reinterpret_cast<const float4 *>(qre + (m0 + c4) * QC + x0);
+                const float4 xi4 = *reinterpret_cast<const float4 *>(qim + (m0 + c4) * QC + x0);
+                const float xr[4] = {xr4.x, xr4.y, xr4.z, xr4.w}, xi[4] = {xi4.x, xi4.y, xi4.z, xi4.w};
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    if (c4 & 1) {
+                        q2r[r][c4 / 2].y = xr[r] - (rr[r][c4 / 2].y - ii[r][c4 / 2].y);
+                        q2i[r][c4 / 2].y = xi[r] - (ri[r][c4 / 2].y + ir[r][c4 / 2].y);
+                    } else {
+                        q2r[r][c4 / 2].x = xr[r] - (rr[r][c4 / 2].x - ii[r][c4 / 2].x);
+                        q2i[r][c4 / 2].x = xi[r] - (ri[r][c4 / 2].x + ir[r][c4 / 2].x);
+                    }
+                }
+            }
+        };
+        auto put = [&](int m0) {
+#pragma unroll
+            for (int h2 = 0; h2 < 2; ++h2) {
+                float *c0 = qre + (m0 + 2 * h2) * QC + x0, *c1 = qim + (m0 + 2 * h2) * QC + x0;
+                *reinterpret_cast<float4 *>(c0) = make_float4(q2r[0][h2].x, q2r[1][h2].x, q2r[2][h2].x, q2r[3][h2].x);
+                *reinterpret_cast<float4 *>(c0 + QC) = make_float4(q2r[0][h2].y, q2r[1][h2].y, q2r[2][h2].y, q2r[3][h2].y);
+                *reinterpret_cast<float4 *>(c1) = make_float4(q2i[0][h2].x, q2i[1][h2].x, q2i[2][h2].x, q2i[3][h2].x);
+                *reinterpret_cast<float4 *>(c1 + QC) = make_float4(q2i[0][h2].y, q2i[1][h2].y, q2i[2][h2].y, q2i[3][h2].y);
+            }
+        };
+        const int w8 = 8 * (t >> 5);
+        block(H2 + 4 * (7 - bj), H2 + 32 - w8);
+        __syncthreads();   // every thread has read the high columns
+        put(H2 + 4 * (7 - bj));
+        block(4 * bj, w8 + 8);
+        __syncthreads();
+        put(4 * bj);
         __syncthreads();
     } else {
         __syncthreads();
