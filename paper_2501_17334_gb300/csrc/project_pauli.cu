@@ -67,6 +67,7 @@ struct PauliShape {
     static constexpr int TPC = NB > 648 ? 648 : NB;          // threads per chain (each takes NB / TPC blocks)
     static constexpr int CPB = Q <= 2 ? 128 : (Q == 3 ? 48 : (Q == 4 ? 8 : 1));   // chains per CTA
     static constexpr int threads = TPC * CPB;                // 128, 128, 288, 288, 216, 648
+    static constexpr int final_lanes = Q <= 3 ? 1 : 32 / CPB;   // per chain, for the sum over its threads (4, 32, 32)
     static constexpr int min_ctas = Q <= 2 ? 8 : (Q <= 4 ? 4 : (Q == 5 ? 5 : 1));   // per SM (a register cap)
     static constexpr int NS = Q == 1 ? 3 : 9;                // settings of the last one or two qubits
     // the setting sums (NS x NB (hi, lo) pairs per chain) take the odd-level buffer when the last
@@ -274,25 +275,39 @@ __global__ void __launch_bounds__(PauliShape<Q>::threads, PauliShape<Q>::min_cta
     acc_lo += extra - (comp.x + comp.y);
     if (xmin < 0x00800000) acc_hi = -INFINITY;
 
-    // the chain's threads' pairs, added in thread order (two-sum of the high parts) by one thread
-    // per chain; the CTA's chains sit in its first threads, so the FP64 result (scarce FP64
-    // instructions, each costing its warp the same however many lanes are active) takes a few
-    // warp instructions per CTA
+    // The chain's threads' pairs, added with two-sums of the high parts: FL lanes per chain take every
+    // FL-th thread's pair in turn and join by shuffles.  (One thread adding all TPC pairs in order, a
+    // dependent chain of 216 at five and 648 at six qubits, was a quarter and almost half of a CTA's
+    // life: 149 -> 124 us for 8192 five-qubit chains, 159 -> 128 for 1024
+    // six-qubit ones.)  The CTA's chains sit in its first threads, so the FP64 result (scarce FP64
+    // instructions, each costing its warp the same however many lanes are active) takes a few warp
+    // instructions per CTA.
     if constexpr (TPC == 1) {
         if (active) a.out[c] = (double)acc_hi + (double)acc_lo;
     } else {
+        constexpr int FL = S::final_lanes;
         part[threadIdx.x] = acc_hi;
         part_lo[threadIdx.x] = acc_lo;
         __syncthreads();
-        if (threadIdx.x < CPB) {
-            const int64_t cc = (int64_t)blockIdx.x * CPB + threadIdx.x;
+        if (threadIdx.x < CPB * FL) {
+            const int fg = threadIdx.x / FL, fl = threadIdx.x % FL;
+            const int64_t cc = (int64_t)blockIdx.x * CPB + fg;
             float hi = 0.0f, lo = 0.0f;
-            for (int t = 0; t < TPC; ++t) {
+            for (int t = fl; t < TPC; t += FL) {
                 float e;
-                two_sum(hi, part[threadIdx.x * TPC + t], hi, e);
-                lo += e + part_lo[threadIdx.x * TPC + t];
+                two_sum(hi, part[fg * TPC + t], hi, e);
+                lo += e + part_lo[fg * TPC + t];
             }
-            if (cc < a.rows) a.out[cc] = (double)hi + (double)lo;
+            if constexpr (FL > 1) {   // (one whole warp)
+#pragma unroll
+                for (int off = FL / 2; off > 0; off >>= 1) {
+                    const float oh = __shfl_down_sync(0xffffffffu, hi, off), ol = __shfl_down_sync(0xffffffffu, lo, off);
+                    float e;
+                    two_sum(hi, oh, hi, e);
+                    lo += e + ol;
+                }
+            }
+            if (fl == 0 && cc < a.rows) a.out[cc] = (double)hi + (double)lo;
         }
     }
 }
