@@ -223,8 +223,8 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
 /* Enqueues num_steps steps j -> j+1 of Algorithm 2 for every chain of every problem
  * (proposal, Algorithm 1, likelihood, accept, adaptation, thinning and pooling).
  * Asynchronous on the handle's stream; resumable (step numbering continues).
- * A step is one small kernel that advances the device-side step counter, then the
- * proposal, projection and accept kernels of every problem.  With use_graph the first
+ * A step is the proposal, projection and accept kernels of every problem; the last of the
+ * accept kernels advances the step counter on the device.  With use_graph the first
  * call captures that sequence once (on private streams, the problems of a handle on up
  * to eight parallel branches, since they are independent) and every step launches the
  * graph; the results are bit-identical to plain launches.  One- and two-qubit problems in the FP32

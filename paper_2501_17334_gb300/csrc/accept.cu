@@ -18,16 +18,18 @@ struct AcceptArgs {
     uint32_t step;     // j
     int kept;          // j is a kept step (j % T == 0 and j > burn_in)
     int64_t kept_idx;  // index of this kept state (0-based) in the trajectories
-    const StepState *step_dev;   // when not null: step, kept and kept_idx come from here
+    StepState *step_dev;         // when not null: step, kept and kept_idx follow from the counter here
+    uint32_t step_ctas;          // and the last of this many CTAs (all accept kernels of the step) advances it
+    int thin, burn_in;
 };
 
 // One CTA owns chains [C b, C b + C) and pool slot b, C = p.accept_cpc <= 128.
 __global__ void __launch_bounds__(kThreads) accept_kernel(AcceptArgs a) {
     const ProblemView &p = a.p;
     if (a.step_dev) {   // (a is this thread's copy of the parameters)
-        a.step = a.step_dev->step;
-        a.kept = a.step_dev->kept;
-        a.kept_idx = a.step_dev->kept_idx;
+        a.step = a.step_dev->step + 1u;
+        a.kept = (a.step % (uint32_t)a.thin == 0u) && ((int64_t)a.step > (int64_t)a.burn_in);
+        a.kept_idx = a.step_dev->kept_count;
     }
     __shared__ uint8_t flag[kChainsPerCta];
     __shared__ float inv_tr[kChainsPerCta];
@@ -101,7 +103,8 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(AcceptArgs a) {
     // ---- phase 2: rho write-back, pooling of the current state, trajectories ------------
     // Thread t moves float4 number (t mod V) of a chain's packed rho (V = d/4 per chain) for
     // the chains t/V, t/V + P, ... (P = 256/V chains in flight per pass, four passes
-    // unrolled so that several independent loads are outstanding).  Pool sums: per-thread
+    // unrolled so that several independent loads are outstanding; eight or sixteen cost registers and
+    // with them occupancy: 34 and 33 against 26 us at 65536 four-qubit chains).  Pool sums: per-thread
     // float4 partials, then a shared-memory reduction over the P chain lanes.
     const int d = p.d;
     const int V = d / 4;
@@ -181,6 +184,17 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(AcceptArgs a) {
             __syncthreads();
         }
         if (V < kThreads) break;
+    }
+    if (a.step_dev) {   // every thread has read the counter: the step's last CTA advances it
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();
+            if (atomicAdd(&a.step_dev->ticket, 1u) == a.step_ctas - 1u) {
+                a.step_dev->ticket = 0u;
+                a.step_dev->step = a.step;
+                a.step_dev->kept_count = a.kept_idx + a.kept;
+            }
+        }
     }
 }
 
@@ -391,34 +405,22 @@ __global__ void inject_nan_kernel(float *y, const uint8_t *cur, int64_t R, int n
     for (int e = threadIdx.x; e < nx; e += blockDim.x) y[((int64_t)b * R + chain) * nx + e] = __int_as_float(0x7fc00000);
 }
 
-// Opens step j = step + 1 (one thread): whether j is kept and at which index.
-__global__ void advance_step_kernel(StepState *st, int thin, int burn_in) {
-    const uint32_t j = st->step + 1u;
-    const int kept = (j % (uint32_t)thin == 0u) && ((int64_t)j > (int64_t)burn_in);
-    st->step = j;
-    st->kept = kept;
-    st->kept_idx = st->kept_count;
-    st->kept_count += kept;
-}
-
 }  // namespace
 
-cudaError_t launch_advance_step(StepState *st, int thin, int burn_in, cudaStream_t s) {
-    advance_step_kernel<<<1, 1, 0, s>>>(st, thin, burn_in);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_accept(const ProblemView &p, const SamplerParams &sp, int mode, const StepState *step_dev, uint32_t step,
-                          bool kept, int64_t kept_idx, uint32_t *status, cudaStream_t s) {
+cudaError_t launch_accept(const ProblemView &p, const SamplerParams &sp, int mode, StepState *step_dev, uint32_t step_ctas,
+                          int thin, int burn_in, uint32_t *status, cudaStream_t s) {
     (void)status;
     AcceptArgs a;
     a.p = p;
     a.sp = sp;
     a.mode = mode;
-    a.step = step;
-    a.kept = kept ? 1 : 0;
-    a.kept_idx = kept_idx;
+    a.step = 0u;
+    a.kept = 0;
+    a.kept_idx = 0;
     a.step_dev = step_dev;
+    a.step_ctas = step_ctas;
+    a.thin = thin;
+    a.burn_in = burn_in;
     const int64_t blocks = (p.R + p.accept_cpc - 1) / p.accept_cpc;
     accept_kernel<<<(unsigned)blocks, kThreads, 0, s>>>(a);
     return cudaGetLastError();

@@ -485,7 +485,10 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
         // smaller sizes; it must hold at least one chain)
         if (cfg->propose_threads != 0 && v.D <= 16 && (v.qr_passes == 0 || v.qr_passes == 3) &&
             cfg->propose_threads >= v.D)
+        {
             v.propose_threads = cfg->propose_threads;
+            v.propose_fixed = true;
+        }
         v.accept_cpc = accept_chains_per_cta(v.R, v.d);
         v.n_slots = (int)((v.R + v.accept_cpc - 1) / v.accept_cpc);
         v.n_diag = (int)std::min<int64_t>(cfg->diag_chains, v.R);
@@ -699,7 +702,7 @@ qst_status enqueue_init(qst_handle *h, HostProblem &hp) {
     st = enqueue_projection(h, hp, v.R, nullptr);
     if (st != QST_OK) return st;
     return launch(h, QST_KERNEL_ACCEPT, "accept (init)", [&] {
-        return launch_accept(v, h->sp, MODE_INIT, nullptr, 0u, false, 0, h->d_status, h->stream);
+        return launch_accept(v, h->sp, MODE_INIT, nullptr, 0u, 1, 0, h->d_status, h->stream);
     });
 }
 
@@ -863,7 +866,7 @@ qst_status autotune_propose(qst_handle *h) {
         ProblemView &v = hp.v;
         if (v.D > 16 || (v.qr_passes != 0 && v.qr_passes != 3) || h->cfg.propose_threads != 0) continue;
         const int64_t blocks128 = (v.R + 128 / v.D - 1) / (128 / v.D);
-        if (blocks128 >= 2 * 5 * (int64_t)sms) continue;
+        if (blocks128 >= 2 * 5 * (int64_t)sms || propose_split(v, v.R)) continue;
         int best = 128;
         float best_ms = 0.0f;
         for (int threads : {128, 64, 32}) {
@@ -1007,12 +1010,12 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
 
 namespace {
 
-// One step's launches on h->stream: open step j on the device, then every problem's
-// proposal, projection and accept, all reading j from the device.  With `branches` (graph
+// One step's launches on h->stream: every problem's proposal, projection and accept, all reading the
+// step from the device, where the last accept CTA advances it.  With `branches` (graph
 // capture) the problems are spread over parallel branches -- they are independent -- so
 // the graph runs the kernels of different problems concurrently.  With `multi` the problems that
 // run many steps per launch (enqueue_multi) are left out.
-qst_status enqueue_problem(qst_handle *h, HostProblem &hp) {
+qst_status enqueue_problem(qst_handle *h, HostProblem &hp, uint32_t step_ctas) {
     ProblemView &v = hp.v;
     qst_status st = launch(h, QST_KERNEL_PROPOSE, "propose", [&] {
         return launch_propose(v, MODE_STEP, 0u, h->d_step, nullptr, 0, uses_tc(v), nullptr, h->d_status, h->stream);
@@ -1021,21 +1024,24 @@ qst_status enqueue_problem(qst_handle *h, HostProblem &hp) {
     st = enqueue_projection(h, hp, v.R, nullptr);
     if (st != QST_OK) return st;
     return launch(h, QST_KERNEL_ACCEPT, "accept", [&] {
-        return launch_accept(v, h->sp, MODE_STEP, h->d_step, 0u, false, 0, h->d_status, h->stream);
+        return launch_accept(v, h->sp, MODE_STEP, h->d_step, step_ctas, h->cfg.thin, h->cfg.burn_in, h->d_status,
+                             h->stream);
     });
 }
 
 qst_status enqueue_step(qst_handle *h, bool branches, bool multi) {
-    qst_status st = launch(h, QST_KERNEL_ACCEPT, "advance step",
-                           [&] { return launch_advance_step(h->d_step, h->cfg.thin, h->cfg.burn_in, h->stream); });
-    if (st != QST_OK) return st;
+    qst_status st = QST_OK;
     std::vector<HostProblem *> probs;
+    uint32_t step_ctas = 0;   // accept CTAs of the step: the last one advances the step counter
     for (auto &hp : h->plan.probs)
-        if (!multi || !fused_supported(hp.v)) probs.push_back(&hp);
+        if (!multi || !fused_supported(hp.v)) {
+            probs.push_back(&hp);
+            step_ctas += (uint32_t)hp.v.n_slots;
+        }
     const int np = (int)probs.size();
     if (!branches || np == 1) {
         for (HostProblem *hp : probs) {
-            st = enqueue_problem(h, *hp);
+            st = enqueue_problem(h, *hp, step_ctas);
             if (st != QST_OK) return st;
         }
         return QST_OK;
@@ -1046,7 +1052,7 @@ qst_status enqueue_step(qst_handle *h, bool branches, bool multi) {
     for (int b = 0; b < nb; ++b) QST_CUDA(cudaStreamWaitEvent(h->branch[b], h->fork_ev, 0), "branch wait");
     for (int i = 0; i < np && st == QST_OK; ++i) {
         h->stream = h->branch[i % nb];
-        st = enqueue_problem(h, *probs[i]);
+        st = enqueue_problem(h, *probs[i], step_ctas);
     }
     h->stream = origin;
     if (st != QST_OK) return st;
@@ -1151,7 +1157,7 @@ qst_status qst_run_chains(qst_handle *h, int64_t num_steps) {
     }
     for (int64_t s = 0; s < num_steps; ++s) {
         const int64_t j = h->steps_done + 1;
-        const bool kept = (j % h->cfg.thin == 0) && (j > h->cfg.burn_in);   // mirrors advance_step_kernel
+        const bool kept = (j % h->cfg.thin == 0) && (j > h->cfg.burn_in);   // as the accept kernel decides it
         if (graph) {
             QST_CUDA(cudaGraphLaunch(h->graph_exec, h->stream), "launch step graph");
             h->launches += h->graph_kernels;
@@ -1278,7 +1284,7 @@ qst_status qst_diagnostics(qst_handle *h, int32_t problem, qst_diag *out, double
                                                                         : h->cfg.precision
                                                  : (int32_t)QST_PREC_FP32;
     out->propose_chains_per_cta =
-        (uint32_t)(v.D <= 16 ? v.propose_threads / v.D : (v.D == 32 ? (v.qr_passes == 3 ? 2 : 4) : 1));
+        (uint32_t)(v.D <= 16 ? (propose_split(v, v.R) ? 32 : v.propose_threads) / v.D : (v.D == 32 ? (v.qr_passes == 3 ? 2 : 4) : 1));
     out->qr_passes = v.qr_passes;
     out->accept_chains_per_cta = (uint32_t)v.accept_cpc;
     if (st != QST_OK) return st;

@@ -596,15 +596,11 @@ __global__ void __launch_bounds__(kPoolThreads) fused_pool_kernel(ProblemView p,
 
 __global__ void snapshot_step_kernel(const StepState *st, StepState *base) { *base = *st; }
 
-// n steps at once: the state after n calls of advance_step_kernel
+// n steps at once, where no per-step kernels run beside
 __global__ void advance_steps_kernel(StepState *st, uint32_t n, int thin, int64_t burn_in) {
     const int64_t j0 = st->step, j1 = j0 + n;
-    const int64_t add = kept_up_to(j1, thin, burn_in) - kept_up_to(j0, thin, burn_in);
-    const bool kept = (j1 % thin == 0) && j1 > burn_in;
     st->step = (uint32_t)j1;
-    st->kept = kept ? 1 : 0;
-    st->kept_idx = st->kept_count + add - (kept ? 1 : 0);
-    st->kept_count += add;
+    st->kept_count += kept_up_to(j1, thin, burn_in) - kept_up_to(j0, thin, burn_in);
 }
 
 template <int D, int PASSES, int LPC, bool PAULI, bool POISSON>

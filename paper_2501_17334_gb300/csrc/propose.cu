@@ -55,7 +55,7 @@ struct ProposeArgs {
     int64_t chain_offset;
     uint64_t seed;
     uint32_t step;
-    const StepState *step_dev;   // MODE_STEP: when not null the step is read from here
+    const StepState *step_dev;   // MODE_STEP: when not null the step is the one after this counter's
     int mode;
     int d_pad;
     Philox::RoundKeys rk;        // the generator's round keys for `seed`
@@ -64,8 +64,19 @@ struct ProposeArgs {
 // THREADS: the CTA size (chains per CTA = THREADS / D); 128 by default, 64 or 32 when the
 // autotuner finds that a small problem covers more SMs that way.  The register budget per
 // thread is the same for every size (five 128-thread CTAs' worth per SM).
-template <int D, int PASSES, int THREADS = kThreads>
-__global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kernel(ProposeArgs a) {
+// 128-thread CTAs per SM the register budget is set for: five (96 registers), at eight lanes per
+// chain seven (72: 65536 three-qubit chains 94 -> 89 us, 16384 29.1 -> 28.1).
+template <int D>
+constexpr int propose_ctas() {
+    return D == 8 ? 7 : 5;
+}
+
+// GRP = 2: two groups of D lanes share a chain.  They take the latent blocks, the refinement's dot
+// products and its update of U, W (at four qubits) and rho's entries in turn, and repeat the sweep
+// and the triangular solve, whose steps depend on one another: the shorter step while there are too
+// few chains to fill the chip (propose_split).
+template <int D, int PASSES, int THREADS = kThreads, int GRP = 1>
+__global__ void __launch_bounds__(THREADS, (GRP == 1 ? propose_ctas<D>() : 5) * kThreads / THREADS) propose_kernel(ProposeArgs a) {
     using S = Shape<D, PASSES, THREADS>;
     constexpr int d = S::d;
     constexpr int nx = 4 * d;
@@ -74,11 +85,13 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
     constexpr int PK = S::pk_stride;
     extern __shared__ __align__(16) float smem[];
 
+    constexpr int LPC = D * GRP;         // lanes per chain
     const int j = threadIdx.x % D;       // owned column (and, in steps 2b and 4, owned row)
-    const int g = threadIdx.x / D;       // chain slot in the block
-    const int64_t c = (int64_t)blockIdx.x * S::chains_per_block + g;
+    const int l = threadIdx.x % LPC, grp = GRP == 1 ? 0 : l / D;
+    const int g = threadIdx.x / LPC;     // chain slot in the block
+    const int64_t c = (int64_t)blockIdx.x * (THREADS / LPC) + g;
     const bool active = c < a.rows;
-    const uint32_t step = (a.step_dev && a.mode == MODE_STEP) ? a.step_dev->step : a.step;
+    const uint32_t step = (a.step_dev && a.mode == MODE_STEP) ? a.step_dev->step + 1u : a.step;
     float *sm = smem + g * S::smem_floats;
     float *qre = sm, *qim = sm + D * QC;                 // Q planes (column stride QC)
     float2 *wsm = reinterpret_cast<float2 *>(sm);        // W row-major (row stride RS), replaces Q
@@ -108,7 +121,7 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
     const float *gsrc = (a.mode == MODE_EVAL) ? a.x_eval + cc * nx : ydst;
     float2 hr[D / 2], hi[D / 2];   // H's column j, entries (2p, 2p + 1) in pair p
     if constexpr (D >= 4) {
-        // A part is d/4 Philox blocks of four entries.  Lane j takes blocks j, j + D, ..: a chain's
+        // A part is d/4 Philox blocks of four entries.  Lane l takes blocks l, l + LPC, ..: a chain's
         // lanes then read and write consecutive 16-byte pieces of y, and H's blocks reach the lanes that own
         // their columns through shared memory (area B where the refinement keeps H's columns
         // anyway, the Q planes otherwise).
@@ -122,19 +135,19 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
         };
 #pragma unroll 1
         for (int part = 0; part < 4; ++part) {
-            const int e0 = part * d + 4 * j;    // element index of this lane's first block
-            float4 y0[D / 4];
+            const int e0 = part * d + 4 * l;    // element index of this lane's first block
+            float4 y0[D / 4 / GRP];
 #pragma unroll
-            for (int q = 0; q < D / 4; ++q) {
+            for (int q = 0; q < D / 4 / GRP; ++q) {
                 y0[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (active && a.mode == MODE_STEP) y0[q] = *reinterpret_cast<const float4 *>(ysrc + e0 + 4 * D * q);
-                if (active && a.mode == MODE_EVAL) y0[q] = *reinterpret_cast<const float4 *>(a.x_eval + cc * nx + e0 + 4 * D * q);
+                if (active && a.mode == MODE_STEP) y0[q] = *reinterpret_cast<const float4 *>(ysrc + e0 + 4 * LPC * q);
+                if (active && a.mode == MODE_EVAL) y0[q] = *reinterpret_cast<const float4 *>(a.x_eval + cc * nx + e0 + 4 * LPC * q);
             }
 #pragma unroll
-            for (int q = 0; q < D / 4; ++q) {
+            for (int q = 0; q < D / 4 / GRP; ++q) {
                 float4 yn = y0[q];
                 if (a.mode != MODE_EVAL) {
-                    const uint4 w = Philox::block(make_uint4((uint32_t)(e0 / 4 + D * q), step, chain_id, tag), a.rk);
+                    const uint4 w = Philox::block(make_uint4((uint32_t)(e0 / 4 + LPC * q), step, chain_id, tag), a.rk);
                     float z0, z1, z2, z3;
                     gaussian_pair_fast(w.x, w.y, z0, z1);
                     gaussian_pair_fast(w.z, w.w, z2, z3);
@@ -142,10 +155,10 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
                     yn.y = __fmaf_rn(coef_y, y0[q].y, coef_eta * z1);
                     yn.z = __fmaf_rn(coef_y, y0[q].z, coef_eta * z2);
                     yn.w = __fmaf_rn(coef_y, y0[q].w, coef_eta * z3);
-                    if (active) *reinterpret_cast<float4 *>(ydst + e0 + 4 * D * q) = yn;
+                    if (active) *reinterpret_cast<float4 *>(ydst + e0 + 4 * LPC * q) = yn;
                 }
-                if (part == 2) stage(hre, qre, j + D * q, yn);
-                if (part == 3) stage(him, qim, j + D * q, yn);
+                if (part == 2) stage(hre, qre, l + LPC * q, yn);
+                if (part == 3) stage(him, qim, l + LPC * q, yn);
             }
         }
         __syncwarp();
@@ -298,8 +311,13 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
         // take the D lanes' results of that step -- element (r, c) at c D + (r ^ c) of the real
         // (hre) and imaginary (him) planes, so that the lanes' writes of a step, a lane's reads
         // of its row and the reads of a column all hit distinct banks.
-        const float ymax = refine_pass<D, QC>(hr, hi, qre, qim, hre, him, rpk, gsrc, j, false, true);
-        if (__any_sync(0xffffffffu, ymax > kRefineTol)) refine_more<D, QC>(qre, qim, hre, him, rpk, gsrc, j, ymax, true);
+        float ymax;
+        if constexpr (GRP == 2)
+            ymax = refine_pass_split<D, QC>(hr, hi, qre, qim, hre, him, rpk, gsrc, j, grp);
+        else
+            ymax = refine_pass<D, QC>(hr, hi, qre, qim, hre, him, rpk, gsrc, j, false, true);
+        if (__any_sync(0xffffffffu, ymax > kRefineTol))
+            refine_more<D, QC>(qre, qim, hre, him, rpk, gsrc, j, ymax, grp == 0);
     }
 
     if constexpr (PASSES == 2) {
@@ -379,18 +397,28 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
         // packed FMAs per row of U instead of sixteen scalar ones.
         float *gsr = sm + S::area_a, *gsi = gsr + D * D;
         {
-            float gr[D], gi[D];
-            if (active) {
-                load_column<D>(gsrc + j * D, gr);
-                load_column<D>(gsrc + d + j * D, gi);
+            if constexpr (GRP == 2) {   // a plane per group
+                float v[D];
+#pragma unroll
+                for (int i = 0; i < D; ++i) v[i] = 0.0f;
+                if (active) load_column<D>(gsrc + grp * d + j * D, v);
+                float *plane = grp ? gsi : gsr;
+#pragma unroll
+                for (int i = 0; i < D; ++i) plane[i * D + j] = v[i];
             } else {
+                float gr[D], gi[D];
+                if (active) {
+                    load_column<D>(gsrc + j * D, gr);
+                    load_column<D>(gsrc + d + j * D, gi);
+                } else {
 #pragma unroll
-                for (int i = 0; i < D; ++i) gr[i] = gi[i] = 0.0f;
-            }
+                    for (int i = 0; i < D; ++i) gr[i] = gi[i] = 0.0f;
+                }
 #pragma unroll
-            for (int i = 0; i < D; ++i) {
-                gsr[i * D + j] = gr[i];
-                gsi[i * D + j] = gi[i];
+                for (int i = 0; i < D; ++i) {
+                    gsr[i * D + j] = gr[i];
+                    gsi[i * D + j] = gi[i];
+                }
             }
         }
         __syncwarp();
@@ -401,9 +429,11 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
         // sums kept apart until the one final add (the assembly's log L error grows with the
         // length of the chains that form W).  The first two rows wait in registers until
         // every lane is done with U, whose storage W takes.
-        float2 wr[4][2], wi[4][2];
+        constexpr int NB = 2 / GRP;   // pairs of rows per lane
+        float2 wr[2 * NB][2], wi[2 * NB][2];
 #pragma unroll
-        for (int hb = 0; hb < 2; ++hb) {
+        for (int nb = 0; nb < NB; ++nb) {
+            const int hb = GRP == 1 ? nb : grp;
             float2 ar[2][2], ai[2][2], xr[2][2], xi[2][2];
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
@@ -442,17 +472,16 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
             for (int r = 0; r < 2; ++r)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    wr[2 * hb + r][h] = __fadd2_rn(ar[r][h], xr[r][h]);
-                    wi[2 * hb + r][h] = __fadd2_rn(ai[r][h], xi[r][h]);
+                    wr[2 * nb + r][h] = __fadd2_rn(ar[r][h], xr[r][h]);
+                    wi[2 * nb + r][h] = __fadd2_rn(ai[r][h], xi[r][h]);
                 }
         }
         __syncwarp();
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {   // W row-major with padded rows (replaces Q)
-            *reinterpret_cast<float4 *>(wsm + (4 * bi + r) * RS + 4 * bj) =
-                make_float4(wr[r][0].x, wi[r][0].x, wr[r][0].y, wi[r][0].y);
-            *reinterpret_cast<float4 *>(wsm + (4 * bi + r) * RS + 4 * bj + 2) =
-                make_float4(wr[r][1].x, wi[r][1].x, wr[r][1].y, wi[r][1].y);
+        for (int r = 0; r < 2 * NB; ++r) {   // W row-major with padded rows (replaces Q)
+            float2 *row = wsm + (4 * bi + (GRP == 1 ? 0 : 2 * grp) + r) * RS + 4 * bj;
+            *reinterpret_cast<float4 *>(row) = make_float4(wr[r][0].x, wi[r][0].x, wr[r][0].y, wi[r][0].y);
+            *reinterpret_cast<float4 *>(row + 2) = make_float4(wr[r][1].x, wi[r][1].x, wr[r][1].y, wi[r][1].y);
         }
         __syncwarp();
     } else {
@@ -525,7 +554,7 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
     // bitwise equal (the same products, accumulated in the same order, negated where the
     // conjugate is taken), so both stores may stand.
 #pragma unroll 1
-    for (int t = 1; t <= D / 2; ++t) {
+    for (int t = 1 + grp; t <= D / 2; t += GRP) {
         const int b = (arow + t) & (D - 1);
         float2 re0 = make_float2(0.f, 0.f), im0 = re0, re1 = re0, im1 = re0;
 #pragma unroll
@@ -543,13 +572,13 @@ __global__ void __launch_bounds__(THREADS, 5 * kThreads / THREADS) propose_kerne
         packed[arow * PK + b] = upper ? re : im;
         packed[b * PK + arow] = upper ? -im : re;
     }
-    if (active && j == 0) a.trace_out[c] = (double)tr_hi + (double)tr_lo;
+    if (active && l == 0) a.trace_out[c] = (double)tr_hi + (double)tr_lo;
     __syncwarp();
 
     // ---- 5. store packed rho (FP32) and its exact bf16 split ----------------------------------
     if (active) {
         float *dst = a.rho_out + c * a.d_pad;
-        for (int e = 4 * j; e < d; e += 4 * D) {
+        for (int e = 4 * l; e < d; e += 4 * LPC) {
             // entries e .. e+3 of the row-major packed rho, staged with row stride PK
             auto staged = [&](int ee) { return packed[(ee / D) * PK + (ee % D)]; };
             const float4 v = make_float4(staged(e), staged(e + 1), staged(e + 2), staged(e + 3));
@@ -677,7 +706,7 @@ __global__ void __launch_bounds__(THREADS, 3 * kThreads / THREADS) propose_kerne
     const int g = threadIdx.x / D;
     const int64_t c = (int64_t)blockIdx.x * S::chains_per_block + g;
     const bool active = c < a.rows;
-    const uint32_t step = (a.step_dev && a.mode == MODE_STEP) ? a.step_dev->step : a.step;
+    const uint32_t step = (a.step_dev && a.mode == MODE_STEP) ? a.step_dev->step + 1u : a.step;
     float *sm = smem + g * S::smem_floats;
     float *qre = sm, *qim = sm + D * QC;                 // Q planes (column stride QC)
     float *wre = sm, *wim = sm + D * QC;                 // W planes (row stride QC), replace Q
@@ -1032,10 +1061,9 @@ __global__ void __launch_bounds__(Wide64::threads, 3) propose_kernel_d64(Propose
     const int t = threadIdx.x;
     const int j = t >> 1, hh = t & 1, r0 = H2 * hh;      // column (or row) j, half hh
     const int r0s = r0 + 4 * hh;                         // where half hh starts within a column (row)
-    const int js = j + 4 * (j >> 5);                     // where entry j sits within a column (row)
     const unsigned pair_mask = 3u << ((t & 31) & ~1);
     const int64_t c = blockIdx.x;                        // one chain per CTA; the grid is exactly rows
-    const uint32_t step = (a.step_dev && a.mode == MODE_STEP) ? a.step_dev->step : a.step;
+    const uint32_t step = (a.step_dev && a.mode == MODE_STEP) ? a.step_dev->step + 1u : a.step;
 
     // ---- 1. latent proposal: this thread's 32 entries of column j of each part -----------------
     float coef_y = 1.0f, coef_eta = 0.0f;
@@ -1368,23 +1396,24 @@ cudaError_t launch_propose_d32(const ProposeArgs &a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-template <int D, int PASSES, int THREADS>
+template <int D, int PASSES, int THREADS, int GRP = 1>
 cudaError_t launch_propose_small(const ProposeArgs &a, int64_t rows, cudaStream_t s) {
     using S = Shape<D, PASSES, THREADS>;
-    const size_t smem = sizeof(float) * S::smem_floats * S::chains_per_block;
+    constexpr int chains = THREADS / (D * GRP);
+    const size_t smem = sizeof(float) * S::smem_floats * chains;
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(propose_kernel<D, PASSES, THREADS>,
+        cudaError_t e = cudaFuncSetAttribute(propose_kernel<D, PASSES, THREADS, GRP>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(propose_kernel<D, PASSES, THREADS>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        e = cudaFuncSetAttribute(propose_kernel<D, PASSES, THREADS, GRP>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    const int64_t blocks = (rows + S::chains_per_block - 1) / S::chains_per_block;
+    const int64_t blocks = (rows + chains - 1) / chains;
     if (blocks == 0) return cudaSuccess;
-    propose_kernel<D, PASSES, THREADS><<<(unsigned)blocks, THREADS, smem, s>>>(a);
+    propose_kernel<D, PASSES, THREADS, GRP><<<(unsigned)blocks, THREADS, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1423,6 +1452,9 @@ cudaError_t launch_propose_pd(const ProblemView &p, int mode, uint32_t step, con
     } else {
         // the CTA sizes the autotuner may pick are built for the default QR (3) and the
         // Hilbert-Schmidt prior (0); other settings run 128-thread CTAs
+        if constexpr (PASSES == 3 && D >= 8) {
+            if (propose_split(p, rows)) return launch_propose_small<D, PASSES, 64, 2>(a, rows, s);
+        }
         if constexpr (PASSES == 0 || PASSES == 3) {
             if (p.propose_threads == 32) return launch_propose_small<D, PASSES, 32>(a, rows, s);
             if (p.propose_threads == 64) return launch_propose_small<D, PASSES, 64>(a, rows, s);
@@ -1441,6 +1473,15 @@ cudaError_t launch_propose_d(const ProblemView &p, int mode, uint32_t step, cons
 }
 
 }  // namespace
+
+// Two groups of lanes per chain (64-thread CTAs) at three and four qubits with the default QR and no
+// CTA size asked for, up to two warps per scheduler at four qubits and one at three.  us at one / two
+// groups: four qubits 64 chains 23.9 / 17.9, 1001 25.1 / 23.7, 2000 31.6 / 34.8; three qubits 64 chains
+// 11.8 / 10.5, 1000 12.5 / 9.8, 2000 11.9 / 12.7.
+bool propose_split(const ProblemView &p, int64_t rows) {
+    if (p.qr_passes != 3 || p.propose_fixed) return false;
+    return (p.D == 16 || p.D == 8) && rows <= 1216;
+}
 
 cudaError_t launch_propose(const ProblemView &p, int mode, uint32_t step, const StepState *step_dev, const float *x_eval,
                            int64_t n_eval, bool want_split, float *rho_norm_out, uint32_t *status, cudaStream_t s) {

@@ -317,9 +317,10 @@ __device__ __noinline__ float refine_tail_rolled(float *qre, float *qim, float *
 
 // The rest of a pass for D <= 16, over registers: the triangular solve on row j of C (area B), Y's
 // upper part and diagonal, U = Q1 - Q1 Y^dag.  `apply`: write this lane's column of the refined U.
-template <int D, int QC>
+// GRP = 2: two groups of D lanes share a chain, and each updates one half of U's rows.
+template <int D, int QC, int GRP = 1>
 __device__ __forceinline__ float refine_tail(float *qre, float *qim, float *hre, float *him, const float2 *rpk, int j,
-                                             float2 mjj, bool apply) {
+                                             float2 mjj, bool apply, int grp = 0) {
     auto cidx = [](int r, int cc) { return cc * D + (r ^ cc); };
     // Y, row j, in registers: y[c] = Y[j][c].  Forward substitution, right-looking: after
     // Y[j][c0] = (M_jc0 - ...) / R_c0c0 every later entry of the row takes its share
@@ -372,8 +373,10 @@ __device__ __forceinline__ float refine_tail(float *qre, float *qim, float *hre,
     // on its own (it is small) and subtracted once.  Rows go in two halves: a half is
     // overwritten only after every lane has read that half of every column.
     constexpr int HP = (D >= 4) ? D / 4 : 1;   // row pairs per half
+    static_assert(GRP == 1 || D >= 4, "halves");
 #pragma unroll
-    for (int half = 0; half < (D >= 4 ? 2 : 1); ++half) {
+    for (int h = 0; h < (D >= 4 && GRP == 1 ? 2 : 1); ++h) {
+        const int half = GRP == 1 ? h : grp;
         float2 cr[HP], ci[HP];
 #pragma unroll
         for (int p = 0; p < HP; ++p) cr[p] = ci[p] = make_float2(0.f, 0.f);
@@ -487,6 +490,29 @@ __device__ __forceinline__ float refine_pass(float2 (&hr)[D / 2], float2 (&hi)[D
         return refine_tail_rolled<D, QC>(qre, qim, hre, him, rpk, j, mjj, apply);
     else
         return refine_tail<D, QC>(qre, qim, hre, him, rpk, j, mjj, apply);
+}
+
+// refine_pass's first pass where two groups of D lanes share a chain: the groups take the entries of
+// row j of C in turn (two of H's columns are freed per step), and half of U's rows each.
+template <int D, int QC>
+__device__ __forceinline__ float refine_pass_split(const float2 (&hr)[D / 2], const float2 (&hi)[D / 2], float *qre,
+                                                   float *qim, float *hre, float *him, const float2 *rpk,
+                                                   const float *gsrc, int j, int grp) {
+    constexpr int d = D * D;
+#pragma unroll 1
+    for (int c2 = 0; c2 < D; c2 += 2) {
+        const int cc = c2 + grp;
+        const bool lower = cc < j;
+        const float2 res = sum_products_exact<D>(hr, hi, lower ? hre + cc * D : qre + cc * QC,
+                                                 lower ? him + cc * D : qim + cc * QC, lower ? 192.0f : 6.0f,
+                                                 cc == j ? 1.0f : 0.0f, lower ? hsw<D, QC>(cc) : qsw<D, QC>(cc));
+        __syncwarp();   // every lane is done with columns c2 and c2 + 1 of H
+        hre[cc * D + (j ^ cc)] = res.x;
+        him[cc * D + (j ^ cc)] = res.y;
+    }
+    const float2 mjj = sum_products_exact<D>(hr, hi, gsrc + 2 * d + j * D, gsrc + 3 * d + j * D, 192.0f, 0.0f);
+    __syncwarp();
+    return refine_tail<D, QC, 2>(qre, qim, hre, him, rpk, j, mjj, true, grp);
 }
 
 // The passes after the first, for the few chains whose first pass left |Y| above kRefineTol: out

@@ -109,14 +109,14 @@ __device__ __forceinline__ float deviance_log(float x) {
     return (__float_as_int(x) >= 0x00800000) ? r : -INFINITY;
 }
 
-// Step counter kept on the device, so that a step's launches have fixed arguments and can
-// be captured once in a CUDA graph: advance_step_kernel opens step j = step + 1 and decides
-// whether it is kept (j % T == 0 and j > burn_in) and at which trajectory index.
+// Step counter kept on the device, so that a step's launches have fixed arguments and can be captured
+// once in a CUDA graph.  The kernels of step j read step = j - 1; the last CTA of the step's accept
+// kernels to finish (counted by `ticket`) advances it.  (A one-thread kernel that opened each step
+// cost a node of the step's dependent chain: 47.1 -> 45.8 us per step at 16384 three-qubit chains.)
 struct StepState {
-    uint32_t step;       // j of the step being run (0 before the first)
-    int32_t kept;        // step j is kept
-    int64_t kept_idx;    // index of step j's state among the kept states
-    int64_t kept_count;  // kept states so far, this step included
+    uint32_t step;       // steps taken
+    uint32_t ticket;     // accept CTAs of the step under way that are done
+    int64_t kept_count;  // kept states so far
 };
 
 // Operand kind of the tensor-core projection (the mixed forms).  TC_BF16X3: rho split into
@@ -183,6 +183,7 @@ struct ProblemView {
     int qr_passes;               // 1 or 2 modified Gram-Schmidt passes, 3: one pass and the refinement; 0: no QR
                                  // (Hilbert-Schmidt prior, W = G)
     int propose_threads = 128;   // CTA size of the proposal kernel at D <= 16 (32, 64 or 128; autotuned)
+    bool propose_fixed = false;  // that size was asked for
 };
 
 struct SamplerParams {
@@ -193,14 +194,16 @@ struct SamplerParams {
 // ---------------------------------------------------------------------------------------
 // Launchers (each returns the CUDA launch error).
 // ---------------------------------------------------------------------------------------
-cudaError_t launch_advance_step(StepState *st, int thin, int burn_in, cudaStream_t s);
-// step_dev: when not null the step is read from it (MODE_STEP), else `step` is used
+// step_dev: when not null the step is the one after it (MODE_STEP), else `step` is used
 cudaError_t launch_propose(const ProblemView &p, int mode, uint32_t step, const StepState *step_dev, const float *x_eval, int64_t n_eval,
                            bool want_split, float *rho_norm_out, uint32_t *status, cudaStream_t s);
+bool propose_split(const ProblemView &p, int64_t rows);   // two groups of lanes per chain (32 / D chains per CTA)
 cudaError_t launch_project_fp32(const ProblemView &p, const float *A, int64_t rows, double *out_part,
                                 float *p_out, cudaStream_t s);
-cudaError_t launch_accept(const ProblemView &p, const SamplerParams &sp, int mode, const StepState *step_dev, uint32_t step, bool kept,
-                          int64_t kept_idx, uint32_t *status, cudaStream_t s);
+// step_dev, MODE_STEP: the counter, which the last of step_ctas accept CTAs (those of all the step's
+// problems; p.n_slots each) advances
+cudaError_t launch_accept(const ProblemView &p, const SamplerParams &sp, int mode, StepState *step_dev, uint32_t step_ctas,
+                          int thin, int burn_in, uint32_t *status, cudaStream_t s);
 cudaError_t launch_pool_reduce(const ProblemView &p, double *out, cudaStream_t s);
 // ACF sums of the diagnostic chains: part [n_diag][acf_slabs(d)][lmax + 1], then acf_raw [n_diag][lmax + 1]
 int acf_slabs(int d);
