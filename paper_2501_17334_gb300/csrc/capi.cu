@@ -948,9 +948,13 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
                                      cudaMemcpyHostToDevice, h->stream), "upload deviance weights");
             QST_CUDA(cudaMemcpyAsync(h->ws + L.pauli_wc, hp.pauli_wc.data(), sizeof(float2) * hp.pauli_wc.size(),
                                      cudaMemcpyHostToDevice, h->stream), "upload counts (pairs)");
-            QST_CUDA(cudaMemcpyAsync(h->ws + L.pauli_perm, hp.pauli_perm.data(),
-                                     sizeof(int32_t) * hp.pauli_perm.size(), cudaMemcpyHostToDevice, h->stream),
-                     "upload tree order");
+            // output-major like the weights, so that a warp reads it coalesced
+            const size_t n = hp.pauli_perm.size(), per = std::min<size_t>(36, n), blocks = n / per;
+            std::vector<int32_t> perm(n);
+            for (size_t o = 0; o < n; ++o) perm[o % per * blocks + o / per] = hp.pauli_perm[o];
+            QST_CUDA(cudaMemcpyAsync(h->ws + L.pauli_perm, perm.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice,
+                                     h->stream), "upload tree order");
+            QST_CUDA(cudaStreamSynchronize(h->stream), "stream sync");   // (perm goes)
         }
         if (!hp.Pbf.empty())
             QST_CUDA(cudaMemcpyAsync(h->ws + L.Ptc, hp.Pbf.data(), sizeof(__nv_bfloat16) * hp.Pbf.size(),

@@ -12,7 +12,7 @@ struct PauliArgs {
     const float *A;          // [rows][d_pad] packed rho
     const float4 *wq;        // [18][6^(Q-2)] (w, w, a, a) of output pair 2 j, 2 j + 1 of block p at [j][p]
     const float2 *wc;        // [18][6^(Q-2)] their counts
-    const int32_t *perm;     // [6^Q] tree order -> setting-major projector index
+    const int32_t *perm;     // [36][6^(Q-2)] output k of block p -> setting-major projector index, at [k][p] (Q = 1: [6])
     const float *ptot;       // [3^Q] shots P_k of setting k
     double *out;             // [rows] the deviance sum (one column group)
     float *p_out;            // [rows][KD] (P_OUT only): p = q / t
@@ -65,8 +65,8 @@ __device__ __forceinline__ void last_split(float e00, float e01, float e10, floa
         if constexpr (P_OUT) {
             if (p_row) {
                 const float h = j < 2 ? 0.5f : 1.0f;
-                p_row[a.perm[o0 + 2 * j]] = h * q2[j].x * inv_t;
-                p_row[a.perm[o0 + 2 * j + 1]] = h * q2[j].y * inv_t;
+                p_row[a.perm[(o0 + 2 * j) * stride + blk]] = h * q2[j].x * inv_t;
+                p_row[a.perm[(o0 + 2 * j + 1) * stride + blk]] = h * q2[j].y * inv_t;
             }
         }
     }

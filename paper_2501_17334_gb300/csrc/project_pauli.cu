@@ -68,7 +68,11 @@ struct PauliShape {
     static constexpr int CPB = Q <= 2 ? 128 : (Q == 3 ? 48 : (Q == 4 ? 8 : 1));   // chains per CTA
     static constexpr int threads = TPC * CPB;                // 128, 128, 288, 288, 216, 648
     static constexpr int final_lanes = Q <= 3 ? 1 : 32 / CPB;   // per chain, for the sum over its threads (4, 32, 32)
-    static constexpr int min_ctas = Q <= 2 ? 8 : (Q <= 4 ? 4 : (Q == 5 ? 5 : 1));   // per SM (a register cap)
+    // per SM (a register cap).  At three qubits two, without spills: 13.6 -> 11.8 us for 5001 chains; at
+    // four the 56 registers of four CTAs win (31.7 against 37.6 us for 10007 chains) unless p is staged
+    static constexpr int min_ctas(bool p_out) {
+        return Q <= 2 ? 8 : Q == 3 ? 2 : Q == 4 ? (p_out ? 2 : 4) : Q == 5 ? 5 : 1;
+    }
     static constexpr int NS = Q == 1 ? 3 : 9;                // settings of the last one or two qubits
     // the setting sums (NS x NB (hi, lo) pairs per chain) take the odd-level buffer when the last
     // stored level is even (Q = 4, 6): it is dead by then
@@ -79,6 +83,12 @@ struct PauliShape {
     static constexpr int bufA = Q == 1 ? 4 : max_level(0);   // even levels (0: the packed rho)
     static constexpr int bufB = cmax(Q >= 3 ? max_level(1) : 0, alias_spart ? 2 * NS * slot_stride : 0);   // odd levels
     static constexpr int floats = (bufA + bufB + 3) / 4 * 4; // per chain
+    // p of a chain is put in setting-major order in shared memory and written out in whole lines up to
+    // five qubits (187 KB a chain at six): straight from the tree's order every store was 4 bytes on its
+    // own, and the order itself read uncoalesced (2000 five-qubit rows 134 -> 58 us, 10007 four-qubit
+    // rows 60 -> 54)
+    static constexpr bool stage_p = Q <= 5;
+    static constexpr int outcomes = ipow(6, Q);
     static_assert(bufA % 4 == 0, "the odd levels' 4 x 4 blocks are read as float4 rows");
     static_assert(NB % TPC == 0, "whole blocks per thread");
 };
@@ -119,7 +129,7 @@ __device__ __forceinline__ void split_level(const float *in, float *out, int par
 }
 
 template <int Q, bool P_OUT, bool POISSON>
-__global__ void __launch_bounds__(PauliShape<Q>::threads, PauliShape<Q>::min_ctas) project_pauli_kernel(PauliArgs a) {
+__global__ void __launch_bounds__(PauliShape<Q>::threads, PauliShape<Q>::min_ctas(P_OUT)) project_pauli_kernel(PauliArgs a) {
     using S = PauliShape<Q>;
     constexpr int D = S::D, d = S::d, TPC = S::TPC, CPB = S::CPB, NB = S::NB;
     constexpr int NS = S::NS;
@@ -179,7 +189,10 @@ __global__ void __launch_bounds__(PauliShape<Q>::threads, PauliShape<Q>::min_cta
     float *p_row = nullptr;
     if constexpr (P_OUT) {
         inv_t = active ? (float)(1.0 / a.trace[c]) : 0.0f;
-        p_row = active ? a.p_out + c * a.KD : nullptr;
+        if constexpr (S::stage_p)
+            p_row = smem + CPB * S::floats + g * S::outcomes;
+        else
+            p_row = active ? a.p_out + c * a.KD : nullptr;
     }
     const float4 ti = tinfo[g];
     // -P_k log(S_k / t) of a setting whose sums are (hi, lo) in units of `unit` q
@@ -228,7 +241,7 @@ __global__ void __launch_bounds__(PauliShape<Q>::threads, PauliShape<Q>::min_cta
 #pragma unroll
             for (int c1 = 0; c1 < 6; ++c1) {
                 last_split<P_OUT>(e00[c1], e01[c1], e10[c1], e11[c1], a, 3 * c1, NB, blk, dev, comp, xmin, sh, sl,
-                                  p_row, 36 * blk + 6 * c1, inv_t);
+                                  p_row, 6 * c1, inv_t);
                 if (c1 & 1) {
 #pragma unroll
                     for (int j = 0; j < 3; ++j) {
@@ -266,6 +279,11 @@ __global__ void __launch_bounds__(PauliShape<Q>::threads, PauliShape<Q>::min_cta
             }
             extra += renorm(vh, vl, slot % 3 < 2 ? 0.5f : 1.0f, k);
         }
+    }
+    if constexpr (P_OUT && S::stage_p) {
+        __syncthreads();
+        if (active)
+            for (int e = lt; e < S::outcomes; e += TPC) a.p_out[c * a.KD + e] = p_row[e];
     }
     // this thread's sum as an unevaluated pair (hi, lo): the two halves of the compensated sum
     // added exactly, the compensations and the small renormalisation terms in lo; a counted
@@ -315,7 +333,7 @@ __global__ void __launch_bounds__(PauliShape<Q>::threads, PauliShape<Q>::min_cta
 template <int Q, bool P_OUT, bool POISSON>
 cudaError_t launch_qpp(const PauliArgs &a, cudaStream_t s) {
     using S = PauliShape<Q>;
-    const size_t smem = sizeof(float) * (size_t)S::floats * S::CPB;
+    const size_t smem = sizeof(float) * (size_t)(S::floats + (P_OUT && S::stage_p ? S::outcomes : 0)) * S::CPB;
     static bool attr_set = false;
     if (!attr_set) {
         const cudaError_t e = cudaFuncSetAttribute(project_pauli_kernel<Q, P_OUT, POISSON>,

@@ -154,7 +154,7 @@ struct ProblemView {
     int pauli;                   // the structured Pauli form of the projection (project_pauli.cu)
     const float4 *pauli_wq;      // [KD / 2] deviance weights per output pair in the structured form's order
     const float2 *pauli_wc;      // [KD / 2] and their counts (pauli_weights)
-    const int32_t *pauli_perm;   // [KD] tree order -> setting-major projector index
+    const int32_t *pauli_perm;   // [KD] tree output k of block p -> setting-major projector index, at [k][p]
 
     // chain state
     float *y;                    // [2][R][nx] double-buffered latent states
