@@ -18,18 +18,20 @@ struct AcceptArgs {
     uint32_t step;     // j
     int kept;          // j is a kept step (j % T == 0 and j > burn_in)
     int64_t kept_idx;  // index of this kept state (0-based) in the trajectories
-    StepState *step_dev;         // when not null: step, kept and kept_idx follow from the counter here
-    uint32_t step_ctas;          // and the last of this many CTAs (all accept kernels of the step) advances it
-    int thin, burn_in;
+    StepState *step_dev; // when not null: step, kept and kept_idx are the open step's, which this closes
 };
 
 // One CTA owns chains [C b, C b + C) and pool slot b, C = p.accept_cpc <= 128.
 __global__ void __launch_bounds__(kThreads) accept_kernel(AcceptArgs a) {
     const ProblemView &p = a.p;
     if (a.step_dev) {   // (a is this thread's copy of the parameters)
-        a.step = a.step_dev->step + 1u;
-        a.kept = (a.step % (uint32_t)a.thin == 0u) && ((int64_t)a.step > (int64_t)a.burn_in);
-        a.kept_idx = a.step_dev->kept_count;
+        a.step = a.step_dev->j;
+        a.kept = a.step_dev->kept;
+        a.kept_idx = a.step_dev->kept_idx;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {   // (no CTA of this launch reads these two)
+            a.step_dev->step = a.step;
+            a.step_dev->kept_count = a.kept_idx + a.kept;
+        }
     }
     __shared__ uint8_t flag[kChainsPerCta];
     __shared__ float inv_tr[kChainsPerCta];
@@ -184,17 +186,6 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(AcceptArgs a) {
             __syncthreads();
         }
         if (V < kThreads) break;
-    }
-    if (a.step_dev) {   // every thread has read the counter: the step's last CTA advances it
-        __syncthreads();
-        if (tid == 0) {
-            __threadfence();
-            if (atomicAdd(&a.step_dev->ticket, 1u) == a.step_ctas - 1u) {
-                a.step_dev->ticket = 0u;
-                a.step_dev->step = a.step;
-                a.step_dev->kept_count = a.kept_idx + a.kept;
-            }
-        }
     }
 }
 
@@ -407,8 +398,8 @@ __global__ void inject_nan_kernel(float *y, const uint8_t *cur, int64_t R, int n
 
 }  // namespace
 
-cudaError_t launch_accept(const ProblemView &p, const SamplerParams &sp, int mode, StepState *step_dev, uint32_t step_ctas,
-                          int thin, int burn_in, uint32_t *status, cudaStream_t s) {
+cudaError_t launch_accept(const ProblemView &p, const SamplerParams &sp, int mode, StepState *step_dev, uint32_t *status,
+                          cudaStream_t s) {
     (void)status;
     AcceptArgs a;
     a.p = p;
@@ -418,9 +409,6 @@ cudaError_t launch_accept(const ProblemView &p, const SamplerParams &sp, int mod
     a.kept = 0;
     a.kept_idx = 0;
     a.step_dev = step_dev;
-    a.step_ctas = step_ctas;
-    a.thin = thin;
-    a.burn_in = burn_in;
     const int64_t blocks = (p.R + p.accept_cpc - 1) / p.accept_cpc;
     accept_kernel<<<(unsigned)blocks, kThreads, 0, s>>>(a);
     return cudaGetLastError();

@@ -123,8 +123,7 @@ struct HostProblem {
 struct Plan {
     std::vector<HostProblem> probs;
     size_t status_off = 0;  // device status word
-    size_t step_off = 0;    // device StepState
-    size_t base_off = 0;    // device StepState: the counter before a qst_run_chains call (multi-step launches)
+    size_t step_off = 0;    // device StepState of every problem
     size_t clear_bytes = 0; // leading bytes that start as zeros
     size_t acf_part_off = 0;   // the ACF's partial sums (one problem's at a time; not chain state)
     size_t bytes = 0;       // total workspace bytes
@@ -533,13 +532,12 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
         L.end = off;
     }
     plan.status_off = take(256);
-    plan.step_off = take(256);
+    plan.step_off = take(sizeof(StepState) * plan.probs.size());
     size_t acf_part = 0;
     for (const auto &hp : plan.probs)
         if (hp.v.n_diag > 0 && hp.v.traj_cap > cfg->acf_lmax)
             acf_part = std::max(acf_part, sizeof(double) * (size_t)hp.v.n_diag * acf_slabs(hp.v.d) * (cfg->acf_lmax + 1));
     plan.acf_part_off = take(acf_part);
-    plan.base_off = take(256);
     plan.clear_bytes = off;   // what follows is written before it is read
     for (auto &hp : plan.probs)
         hp.hist_off = take(sizeof(float) * (size_t)fused_kept_steps(hp.v) * hp.v.R * hp.v.d);
@@ -568,8 +566,7 @@ struct qst_handle {
     size_t ws_bytes = 0;
     bool own_ws = false;
     uint32_t *d_status = nullptr;
-    StepState *d_step = nullptr;
-    StepState *d_base = nullptr;
+    StepState *d_step = nullptr;   // one per problem
     cudaStream_t capture_stream = nullptr;   // private stream the step graph is captured on
     static constexpr int kBranches = 8;      // problems of a graph step run on up to 8 parallel branches
     cudaStream_t branch[kBranches] = {};
@@ -702,7 +699,7 @@ qst_status enqueue_init(qst_handle *h, HostProblem &hp) {
     st = enqueue_projection(h, hp, v.R, nullptr);
     if (st != QST_OK) return st;
     return launch(h, QST_KERNEL_ACCEPT, "accept (init)", [&] {
-        return launch_accept(v, h->sp, MODE_INIT, nullptr, 0u, 1, 0, h->d_status, h->stream);
+        return launch_accept(v, h->sp, MODE_INIT, nullptr, h->d_status, h->stream);
     });
 }
 
@@ -902,6 +899,24 @@ qst_status autotune_propose(qst_handle *h) {
     return st;
 }
 
+StepState *step_of(qst_handle *h, const HostProblem &hp) { return h->d_step + (&hp - h->plan.probs.data()); }
+
+// Every problem's step counter from the handle's.
+qst_status write_steps(qst_handle *h) {
+    std::vector<StepState> ss(h->plan.probs.size());
+    for (size_t i = 0; i < ss.size(); ++i) {
+        ss[i].step = (uint32_t)h->steps_done;
+        ss[i].multi = fused_supported(h->plan.probs[i].v) ? 1u : 0u;
+        ss[i].kept_count = h->kept;
+        ss[i].thin = h->cfg.thin;
+        ss[i].burn_in = h->cfg.burn_in;
+    }
+    QST_CUDA(cudaMemcpyAsync(h->d_step, ss.data(), sizeof(StepState) * ss.size(), cudaMemcpyHostToDevice, h->stream),
+             "write step counters");
+    QST_CUDA(cudaStreamSynchronize(h->stream), "stream sync");
+    return QST_OK;
+}
+
 }  // namespace
 
 qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, const qst_sampler_cfg *cfg,
@@ -936,7 +951,6 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
     QST_CUDA(cudaMemsetAsync(h->ws, 0, h->plan.clear_bytes, h->stream), "clear workspace");
     h->d_status = reinterpret_cast<uint32_t *>(h->ws + h->plan.status_off);
     h->d_step = reinterpret_cast<StepState *>(h->ws + h->plan.step_off);
-    h->d_base = reinterpret_cast<StepState *>(h->ws + h->plan.base_off);
     for (auto &hp : h->plan.probs) {
         bind_problem(h.get(), hp);
         ProblemView &v = hp.v;
@@ -1008,6 +1022,8 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
         if (st == QST_OK) st = autotune_propose(h.get());
         if (st != QST_OK) return st;
     }
+    st = write_steps(h.get());
+    if (st != QST_OK) return st;
     *out = h.release();
     return QST_OK;
 }
@@ -1015,37 +1031,33 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
 namespace {
 
 // One step's launches on h->stream: every problem's proposal, projection and accept, all reading the
-// step from the device, where the last accept CTA advances it.  With `branches` (graph
+// step from the device, where the proposal opens and the accept closes it.  With `branches` (graph
 // capture) the problems are spread over parallel branches -- they are independent -- so
 // the graph runs the kernels of different problems concurrently.  With `multi` the problems that
 // run many steps per launch (enqueue_multi) are left out.
-qst_status enqueue_problem(qst_handle *h, HostProblem &hp, uint32_t step_ctas) {
+qst_status enqueue_problem(qst_handle *h, HostProblem &hp) {
     ProblemView &v = hp.v;
+    StepState *step = step_of(h, hp);
     qst_status st = launch(h, QST_KERNEL_PROPOSE, "propose", [&] {
-        return launch_propose(v, MODE_STEP, 0u, h->d_step, nullptr, 0, uses_tc(v), nullptr, h->d_status, h->stream);
+        return launch_propose(v, MODE_STEP, 0u, step, nullptr, 0, uses_tc(v), nullptr, h->d_status, h->stream);
     });
     if (st != QST_OK) return st;
     st = enqueue_projection(h, hp, v.R, nullptr);
     if (st != QST_OK) return st;
     return launch(h, QST_KERNEL_ACCEPT, "accept", [&] {
-        return launch_accept(v, h->sp, MODE_STEP, h->d_step, step_ctas, h->cfg.thin, h->cfg.burn_in, h->d_status,
-                             h->stream);
+        return launch_accept(v, h->sp, MODE_STEP, step, h->d_status, h->stream);
     });
 }
 
 qst_status enqueue_step(qst_handle *h, bool branches, bool multi) {
     qst_status st = QST_OK;
     std::vector<HostProblem *> probs;
-    uint32_t step_ctas = 0;   // accept CTAs of the step: the last one advances the step counter
     for (auto &hp : h->plan.probs)
-        if (!multi || !fused_supported(hp.v)) {
-            probs.push_back(&hp);
-            step_ctas += (uint32_t)hp.v.n_slots;
-        }
+        if (!multi || !fused_supported(hp.v)) probs.push_back(&hp);
     const int np = (int)probs.size();
     if (!branches || np == 1) {
         for (HostProblem *hp : probs) {
-            st = enqueue_problem(h, *hp, step_ctas);
+            st = enqueue_problem(h, *hp);
             if (st != QST_OK) return st;
         }
         return QST_OK;
@@ -1056,7 +1068,7 @@ qst_status enqueue_step(qst_handle *h, bool branches, bool multi) {
     for (int b = 0; b < nb; ++b) QST_CUDA(cudaStreamWaitEvent(h->branch[b], h->fork_ev, 0), "branch wait");
     for (int i = 0; i < np && st == QST_OK; ++i) {
         h->stream = h->branch[i % nb];
-        st = enqueue_problem(h, *probs[i], step_ctas);
+        st = enqueue_problem(h, *probs[i]);
     }
     h->stream = origin;
     if (st != QST_OK) return st;
@@ -1074,14 +1086,15 @@ qst_status enqueue_multi(qst_handle *h, HostProblem &hp, int64_t num_steps, cuda
     const int64_t burn = h->cfg.burn_in;
     const int64_t most = std::min<int64_t>(1024, (int64_t)fused_kept_steps(hp.v) * thin);
     float *hist = reinterpret_cast<float *>(h->ws + hp.hist_off);
+    const StepState *step = step_of(h, hp);
     for (int64_t off = 0; off < num_steps; off += most) {
         const int n = (int)std::min<int64_t>(most, num_steps - off);
         qst_status st = launch(h, QST_KERNEL_PROPOSE, "steps", [&] {
-            return launch_fused_steps(hp.v, h->sp, h->d_base, (uint32_t)off, n, thin, burn, hist, s);
+            return launch_fused_steps(hp.v, h->sp, step, (uint32_t)off, n, thin, burn, hist, s);
         });
         if (st != QST_OK) return st;
         st = launch(h, QST_KERNEL_ACCEPT, "pool steps", [&] {
-            return launch_fused_pool(hp.v, h->d_base, (uint32_t)off, n, thin, burn, hist, s);
+            return launch_fused_pool(hp.v, step, (uint32_t)off, n, thin, burn, hist, s);
         });
         if (st != QST_OK) return st;
     }
@@ -1145,9 +1158,7 @@ qst_status qst_run_chains(qst_handle *h, int64_t num_steps) {
     }
     int forked = 0;
     if (!multi.empty()) {
-        qst_status st = launch(h, QST_KERNEL_ACCEPT, "snapshot step",
-                               [&] { return launch_snapshot_step(h->d_step, h->d_base, h->stream); });
-        if (st != QST_OK) return st;
+        qst_status st = QST_OK;
         if (steps || multi.size() > 1) {   // on their own branches, beside the other problems
             st = create_branches(h);
             if (st != QST_OK) return st;
@@ -1172,17 +1183,14 @@ qst_status qst_run_chains(qst_handle *h, int64_t num_steps) {
         h->steps_done = j;
         if (kept) h->kept += 1;
     }
-    if (!steps) {
-        qst_status st = launch(h, QST_KERNEL_ACCEPT, "advance steps", [&] {
-            return launch_advance_steps(h->d_step, (uint32_t)num_steps, h->cfg.thin, h->cfg.burn_in, h->stream);
-        });
-        if (st != QST_OK) return st;
-    }
     for (int b = 0; b < forked; ++b) {
         QST_CUDA(cudaEventRecord(h->join_ev[b], h->branch[b]), "join");
         QST_CUDA(cudaStreamWaitEvent(h->stream, h->join_ev[b], 0), "join wait");
     }
-    return QST_OK;
+    if (multi.empty()) return QST_OK;
+    return launch(h, QST_KERNEL_ACCEPT, "advance steps", [&] {   // (their launches have all read the counters)
+        return launch_advance_steps(h->d_step, (int)h->plan.probs.size(), (uint32_t)num_steps, h->stream);
+    });
 }
 
 static qst_status get_problem(qst_handle *h, int32_t problem, HostProblem **hp) {
@@ -1446,10 +1454,8 @@ qst_status qst_restore(qst_handle *h, const void *buffer, size_t bytes) {
     }
     h->steps_done = steps;
     h->kept = kept;
-    StepState ss{};
-    ss.step = (uint32_t)steps;
-    ss.kept_count = kept;
-    QST_CUDA(cudaMemcpy(h->d_step, &ss, sizeof(ss), cudaMemcpyHostToDevice), "restore step counter");
+    st = write_steps(h);
+    if (st != QST_OK) return st;
     return check_status(h);
 }
 

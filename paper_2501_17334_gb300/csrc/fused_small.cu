@@ -38,7 +38,7 @@ constexpr int kSettingSlots = 4;   // settings per D lanes: up to 4 D of them (a
 struct FusedArgs {
     ProblemView p;
     SamplerParams sp;
-    const StepState *base;   // the step counter before the first launch of this call
+    const StepState *base;   // the problem's step counter, as it was before this call
     uint32_t off;            // steps of earlier launches of this call
     int nsteps;
     int thin;
@@ -594,13 +594,15 @@ __global__ void __launch_bounds__(kPoolThreads) fused_pool_kernel(ProblemView p,
     if (threadIdx.x < d && n > 0) slot[e] = acc;
 }
 
-__global__ void snapshot_step_kernel(const StepState *st, StepState *base) { *base = *st; }
-
-// n steps at once, where no per-step kernels run beside
-__global__ void advance_steps_kernel(StepState *st, uint32_t n, int thin, int64_t burn_in) {
-    const int64_t j0 = st->step, j1 = j0 + n;
-    st->step = (uint32_t)j1;
-    st->kept_count += kept_up_to(j1, thin, burn_in) - kept_up_to(j0, thin, burn_in);
+constexpr int kAdvanceThreads = 128;
+__global__ void __launch_bounds__(kAdvanceThreads) advance_steps_kernel(StepState *st, int count, uint32_t n) {
+    for (int i = threadIdx.x; i < count; i += kAdvanceThreads) {
+        StepState &q = st[i];
+        if (!q.multi) continue;
+        const int64_t j0 = q.step, j1 = j0 + n;
+        q.step = (uint32_t)j1;
+        q.kept_count += kept_up_to(j1, (int)q.thin, q.burn_in) - kept_up_to(j0, (int)q.thin, q.burn_in);
+    }
 }
 
 template <int D, int PASSES, int LPC, bool PAULI, bool POISSON>
@@ -687,13 +689,8 @@ cudaError_t launch_fused_pool(const ProblemView &p, const StepState *base, uint3
     return cudaGetLastError();
 }
 
-cudaError_t launch_snapshot_step(const StepState *st, StepState *base, cudaStream_t s) {
-    snapshot_step_kernel<<<1, 1, 0, s>>>(st, base);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_advance_steps(StepState *st, uint32_t n, int thin, int64_t burn_in, cudaStream_t s) {
-    advance_steps_kernel<<<1, 1, 0, s>>>(st, n, thin, burn_in);
+cudaError_t launch_advance_steps(StepState *st, int count, uint32_t n, cudaStream_t s) {
+    advance_steps_kernel<<<1, kAdvanceThreads, 0, s>>>(st, count, n);
     return cudaGetLastError();
 }
 

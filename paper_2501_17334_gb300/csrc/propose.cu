@@ -55,7 +55,7 @@ struct ProposeArgs {
     int64_t chain_offset;
     uint64_t seed;
     uint32_t step;
-    const StepState *step_dev;   // MODE_STEP: when not null the step is the one after this counter's
+    StepState *step_dev;         // MODE_STEP: when not null the step is the one after this counter's, opened here
     int mode;
     int d_pad;
     Philox::RoundKeys rk;        // the generator's round keys for `seed`
@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(THREADS, (GRP == 1 ? propose_ctas<D>() : 5) * 
     const int64_t c = (int64_t)blockIdx.x * (THREADS / LPC) + g;
     const bool active = c < a.rows;
     const uint32_t step = (a.step_dev && a.mode == MODE_STEP) ? a.step_dev->step + 1u : a.step;
+    if (a.step_dev && a.mode == MODE_STEP && blockIdx.x == 0 && threadIdx.x == 0) open_step(a.step_dev);
     float *sm = smem + g * S::smem_floats;
     float *qre = sm, *qim = sm + D * QC;                 // Q planes (column stride QC)
     float2 *wsm = reinterpret_cast<float2 *>(sm);        // W row-major (row stride RS), replaces Q
@@ -707,6 +708,7 @@ __global__ void __launch_bounds__(THREADS, 3 * kThreads / THREADS) propose_kerne
     const int64_t c = (int64_t)blockIdx.x * S::chains_per_block + g;
     const bool active = c < a.rows;
     const uint32_t step = (a.step_dev && a.mode == MODE_STEP) ? a.step_dev->step + 1u : a.step;
+    if (a.step_dev && a.mode == MODE_STEP && blockIdx.x == 0 && threadIdx.x == 0) open_step(a.step_dev);
     float *sm = smem + g * S::smem_floats;
     float *qre = sm, *qim = sm + D * QC;                 // Q planes (column stride QC)
     float *wre = sm, *wim = sm + D * QC;                 // W planes (row stride QC), replace Q
@@ -1064,6 +1066,7 @@ __global__ void __launch_bounds__(Wide64::threads, 3) propose_kernel_d64(Propose
     const unsigned pair_mask = 3u << ((t & 31) & ~1);
     const int64_t c = blockIdx.x;                        // one chain per CTA; the grid is exactly rows
     const uint32_t step = (a.step_dev && a.mode == MODE_STEP) ? a.step_dev->step + 1u : a.step;
+    if (a.step_dev && a.mode == MODE_STEP && blockIdx.x == 0 && threadIdx.x == 0) open_step(a.step_dev);
 
     // ---- 1. latent proposal: this thread's 32 entries of column j of each part -----------------
     float coef_y = 1.0f, coef_eta = 0.0f;
@@ -1418,7 +1421,7 @@ cudaError_t launch_propose_small(const ProposeArgs &a, int64_t rows, cudaStream_
 }
 
 template <int D, int PASSES>
-cudaError_t launch_propose_pd(const ProblemView &p, int mode, uint32_t step, const StepState *step_dev,
+cudaError_t launch_propose_pd(const ProblemView &p, int mode, uint32_t step, StepState *step_dev,
                               const float *x_eval, int64_t rows, bool want_split, float *rho_norm_out, cudaStream_t s) {
     ProposeArgs a;
     a.x_eval = x_eval;
@@ -1464,7 +1467,7 @@ cudaError_t launch_propose_pd(const ProblemView &p, int mode, uint32_t step, con
 }
 
 template <int D>
-cudaError_t launch_propose_d(const ProblemView &p, int mode, uint32_t step, const StepState *step_dev, const float *x_eval,
+cudaError_t launch_propose_d(const ProblemView &p, int mode, uint32_t step, StepState *step_dev, const float *x_eval,
                              int64_t rows, bool want_split, float *rho_norm_out, cudaStream_t s) {
     if (p.qr_passes == 0) return launch_propose_pd<D, 0>(p, mode, step, step_dev, x_eval, rows, want_split, rho_norm_out, s);
     if (p.qr_passes == 1) return launch_propose_pd<D, 1>(p, mode, step, step_dev, x_eval, rows, want_split, rho_norm_out, s);
@@ -1483,7 +1486,7 @@ bool propose_split(const ProblemView &p, int64_t rows) {
     return (p.D == 16 || p.D == 8) && rows <= 1216;
 }
 
-cudaError_t launch_propose(const ProblemView &p, int mode, uint32_t step, const StepState *step_dev, const float *x_eval,
+cudaError_t launch_propose(const ProblemView &p, int mode, uint32_t step, StepState *step_dev, const float *x_eval,
                            int64_t n_eval, bool want_split, float *rho_norm_out, uint32_t *status, cudaStream_t s) {
     (void)status;
     const int64_t rows = (mode == MODE_EVAL) ? n_eval : p.R;

@@ -109,15 +109,30 @@ __device__ __forceinline__ float deviance_log(float x) {
     return (__float_as_int(x) >= 0x00800000) ? r : -INFINITY;
 }
 
-// Step counter kept on the device, so that a step's launches have fixed arguments and can be captured
-// once in a CUDA graph.  The kernels of step j read step = j - 1; the last CTA of the step's accept
-// kernels to finish (counted by `ticket`) advances it.  (A one-thread kernel that opened each step
-// cost a node of the step's dependent chain: 47.1 -> 45.8 us per step at 16384 three-qubit chains.)
+// A problem's step counter, kept on the device so that a step's launches have fixed arguments and can
+// be captured once in a CUDA graph.  The proposal of step j reads step = j - 1, and its first CTA
+// opens the step (j, kept, kept_idx); the accept kernel reads those, and its first CTA closes it (step,
+// kept_count).  So neither kernel writes what its own CTAs read, and the order of the launches is all
+// the ordering there is.  (A one-thread kernel that opened each step was a node of its dependent
+// chain, and advancing the counter in the last accept CTA to finish, by tickets, cost that kernel a
+// fence and an atomic's round trip after its last store.  us per step, those two and this: 2567
+// three-qubit chains 28.7, 26.7, 24.7; 2885 four-qubit chains 35.9, 35.9, 33.9; 1711 one-qubit chains
+// on the tensor cores 18.7, 19.4, 17.5; 16384 three-qubit chains 47.1, 45.8, 45.5.)
 struct StepState {
     uint32_t step;       // steps taken
-    uint32_t ticket;     // accept CTAs of the step under way that are done
+    uint32_t multi;      // the problem runs many steps per launch (advanced by launch_advance_steps)
     int64_t kept_count;  // kept states so far
+    uint32_t j;          // the step under way
+    int32_t kept;        // it is kept (j % T == 0 and j > burn_in)
+    int64_t kept_idx;    // and its index among the kept states (0-based)
+    int64_t thin, burn_in;
 };
+__device__ __forceinline__ void open_step(StepState *st) {
+    const uint32_t j = st->step + 1u;
+    st->j = j;
+    st->kept = (j % (uint32_t)st->thin == 0u) && ((int64_t)j > st->burn_in);
+    st->kept_idx = st->kept_count;
+}
 
 // Operand kind of the tensor-core projection (the mixed forms).  TC_BF16X3: rho split into
 // bf16 hi + mid + lo, P in bf16 (kind::f16).  TC_TF32: rho rounded to TF32 once, P in TF32
@@ -194,16 +209,15 @@ struct SamplerParams {
 // ---------------------------------------------------------------------------------------
 // Launchers (each returns the CUDA launch error).
 // ---------------------------------------------------------------------------------------
-// step_dev: when not null the step is the one after it (MODE_STEP), else `step` is used
-cudaError_t launch_propose(const ProblemView &p, int mode, uint32_t step, const StepState *step_dev, const float *x_eval, int64_t n_eval,
+// step_dev: when not null the step is the one after it (MODE_STEP) and is opened, else `step` is used
+cudaError_t launch_propose(const ProblemView &p, int mode, uint32_t step, StepState *step_dev, const float *x_eval, int64_t n_eval,
                            bool want_split, float *rho_norm_out, uint32_t *status, cudaStream_t s);
 bool propose_split(const ProblemView &p, int64_t rows);   // two groups of lanes per chain (32 / D chains per CTA)
 cudaError_t launch_project_fp32(const ProblemView &p, const float *A, int64_t rows, double *out_part,
                                 float *p_out, cudaStream_t s);
-// step_dev, MODE_STEP: the counter, which the last of step_ctas accept CTAs (those of all the step's
-// problems; p.n_slots each) advances
-cudaError_t launch_accept(const ProblemView &p, const SamplerParams &sp, int mode, StepState *step_dev, uint32_t step_ctas,
-                          int thin, int burn_in, uint32_t *status, cudaStream_t s);
+// step_dev, MODE_STEP: the counter whose open step this closes
+cudaError_t launch_accept(const ProblemView &p, const SamplerParams &sp, int mode, StepState *step_dev, uint32_t *status,
+                          cudaStream_t s);
 cudaError_t launch_pool_reduce(const ProblemView &p, double *out, cudaStream_t s);
 // ACF sums of the diagnostic chains: part [n_diag][acf_slabs(d)][lmax + 1], then acf_raw [n_diag][lmax + 1]
 int acf_slabs(int d);
@@ -214,8 +228,8 @@ cudaError_t launch_philox_blocks(uint64_t seed, uint32_t step, uint32_t tag, uin
                                  uint32_t block0, int32_t nblocks, uint32_t *out, cudaStream_t s);
 cudaError_t launch_inject_nan(const ProblemView &p, int64_t chain, cudaStream_t s);
 
-// Many steps of a one- or two-qubit problem in one launch (fused_small.cu).  `base`: the step counter
-// before the first launch of a qst_run_chains call, `off` the steps of its earlier launches; the
+// Many steps of a one- or two-qubit problem in one launch (fused_small.cu).  `base`: the problem's step
+// counter, as it was before the qst_run_chains call, `off` the steps of its earlier launches; the
 // launch covers nsteps steps with at most fused_kept_steps(p) kept ones, whose states go to `hist`
 // ([kept step][R][d] floats) for launch_fused_pool.
 bool fused_supported(const ProblemView &p);
@@ -224,8 +238,8 @@ cudaError_t launch_fused_steps(const ProblemView &p, const SamplerParams &sp, co
                                int nsteps, int thin, int64_t burn_in, float *hist, cudaStream_t s);
 cudaError_t launch_fused_pool(const ProblemView &p, const StepState *base, uint32_t off, int nsteps, int thin,
                               int64_t burn_in, const float *hist, cudaStream_t s);
-cudaError_t launch_snapshot_step(const StepState *st, StepState *base, cudaStream_t s);
-cudaError_t launch_advance_steps(StepState *st, uint32_t n, int thin, int64_t burn_in, cudaStream_t s);
+// n steps at once for those of the `count` problems that run many steps per launch
+cudaError_t launch_advance_steps(StepState *st, int count, uint32_t n, cudaStream_t s);
 
 // tcgen05 projection in the view's tc_kind (sm_103a).  Returns cudaErrorNotSupported if the
 // shape is outside what the kernel handles.
