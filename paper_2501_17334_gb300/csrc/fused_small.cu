@@ -6,7 +6,7 @@
 // Chains never interact, so here the lanes of a chain run whole steps on their own: the latent
 // state, rho and the chain's scalars stay in registers, the small matrices in a few hundred bytes
 // of shared memory, and nothing but warp barriers orders a step.  A CTA is one warp, so that few
-// chains spread over many SMs: 1.8 us per step for 64 one-qubit chains, 4.8 us for 4096 two-qubit
+// chains spread over many SMs: 1.6 us per step for 64 one-qubit chains, 4.7 us for 4096 two-qubit
 // chains.  Every value is formed by the same operations in the
 // same order as in the per-step kernels, so the chains are the same bits.
 //
