@@ -43,12 +43,12 @@ WORKLOAD = ("config 4: 4-qubit Pauli QST (D=16, 81 bases x 16 outcomes = 1296 pr
 NCU_TRAFFIC = {
     # profiles/propose_kernel_config4.md
     "propose": {"source": "paper_2501_17334_gb300/csrc/propose.cu",
-                "sha256": "8c10ac52736ae4c95d48aa85a8f92c4c6980c58d0d6d7839ae7fbc33d7af46a4",
-                "chains": 32768, "bytes": 135.274752e6 + 166.74688e6},
+                "sha256": "2fb35f57c9ef3a07e38ae82acda70f32930707cb1dfc3eec02eedc7c89bfc618",
+                "chains": 32768, "bytes": 137.376768e6 + 168.585472e6},
     # profiles/project_tc_kernel_config4.md
     "project": {"source": "paper_2501_17334_gb300/csrc/project_tc.cu",
-                "sha256": "37119239961d9995f5809f45982402867e875058dcd74658ffb9b5d6b4a08518",
-                "chains": 32768, "bytes": 51.399424e6 + 25.088e6},
+                "sha256": "db5db012f46a894fd5b3793ee990c3d2d63468449643e6afb93cff51de19ec99",
+                "chains": 32768, "bytes": 51.39968e6 + 0.005376e6},
 }
 
 def _sha256(path):
