@@ -367,12 +367,12 @@ __global__ void __launch_bounds__(kWarp, kMinCtas) fused_small_kernel(const __gr
                     him[cc1 * D + (j ^ cc1)] = res[i].y;
                 }
                 __syncwarp();
-                ymax = refine_tail<D, QC>(qre, qim, hre, him, rpk, j, mjj, own);
+                ymax = refine_tail<D, QC, true>(qre, qim, hre, him, rpk, j, mjj, own);
             } else {
                 ymax = refine_pass<D, QC>(hr, hi, qre, qim, hre, him, rpk, ysm, j, false, true);
             }
             if (__any_sync(0xffffffffu, ymax > kRefineTol))
-                refine_more<D, QC>(qre, qim, hre, him, rpk, ysm, j, ymax, own);
+                refine_more<D, QC, (GRP > 1)>(qre, qim, hre, him, rpk, ysm, j, ymax, own);
         }
         // ---- W = (U + I) G and rho = W W^dag / Tr (steps 3, 4) ----
         float wr[D], wi[D];

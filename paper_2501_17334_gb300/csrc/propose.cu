@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(THREADS, (GRP == 1 ? propose_ctas<D>() : 5) * 
         else
             ymax = refine_pass<D, QC>(hr, hi, qre, qim, hre, him, rpk, gsrc, j, false, true);
         if (__any_sync(0xffffffffu, ymax > kRefineTol))
-            refine_more<D, QC>(qre, qim, hre, him, rpk, gsrc, j, ymax, grp == 0);
+            refine_more<D, QC, (GRP > 1)>(qre, qim, hre, him, rpk, gsrc, j, ymax, grp == 0);
     }
 
     if constexpr (PASSES == 2) {
@@ -845,7 +845,7 @@ __global__ void __launch_bounds__(THREADS, 3 * kThreads / THREADS) propose_kerne
         // error-free M and N rows per lane, the triangular solve, U = Q1 - Q1 Y^dag, repeated while
         // the chain's largest |Y| entry exceeds kRefineTol) ----------------------------------------
         const float ymax = refine_pass<D, QC>(hr, hi, qre, qim, hre, him, rpk, gsrc, j, false, true);
-        if (__any_sync(0xffffffffu, ymax > kRefineTol)) refine_more<D, QC>(qre, qim, hre, him, rpk, gsrc, j, ymax, true);
+        if (__any_sync(0xffffffffu, ymax > kRefineTol)) refine_more<D, QC, false>(qre, qim, hre, him, rpk, gsrc, j, ymax, true);
     }
 
     if constexpr (PASSES == 2) {

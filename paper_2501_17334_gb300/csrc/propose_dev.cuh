@@ -317,8 +317,9 @@ __device__ __noinline__ float refine_tail_rolled(float *qre, float *qim, float *
 
 // The rest of a pass for D <= 16, over registers: the triangular solve on row j of C (area B), Y's
 // upper part and diagonal, U = Q1 - Q1 Y^dag.  `apply`: write this lane's column of the refined U.
-// GRP = 2: two groups of D lanes share a chain, and each updates one half of U's rows.
-template <int D, int QC, int GRP = 1>
+// GRP = 2: two groups of D lanes share a chain, and each updates one half of U's rows.  SHARED: more
+// than one lane holds row j, so the solved entries replace M's only after all of them have read those.
+template <int D, int QC, bool SHARED, int GRP = 1>
 __device__ __forceinline__ float refine_tail(float *qre, float *qim, float *hre, float *him, const float2 *rpk, int j,
                                              float2 mjj, bool apply, int grp = 0) {
     auto cidx = [](int r, int cc) { return cc * D + (r ^ cc); };
@@ -350,6 +351,7 @@ __device__ __forceinline__ float refine_tail(float *qre, float *qim, float *hre,
     }
     const float2 ydiag = make_float2(0.5f * hre[cidx(j, j)], ydi * rpk[j * (j + 1) / 2 + j].y);
     // upper part: Y[j][c] = N_jc - conj(Y[c][j]), c > j, through area B
+    if constexpr (SHARED) __syncwarp();   // the lanes that share this row have read it
 #pragma unroll
     for (int c = 0; c < D - 1; ++c)
         if (c < j) {
@@ -445,9 +447,9 @@ __device__ __forceinline__ float refine_tail(float *qre, float *qim, float *hre,
 // method is described).  `again`: a pass after the first, which reads H's column j back from y'
 // into area B (it held C) and U's column j as this lane's vector; `apply`: write the refined U
 // (a further pass runs for the whole warp when any of its chains needs it, and the others
-// discard theirs, so a chain's bits never depend on its neighbours).  Returns the chain's
-// largest |Y| entry.
-template <int D, int QC>
+// discard theirs, so a chain's bits never depend on its neighbours).  SHARED as in refine_tail.
+// Returns the chain's largest |Y| entry.
+template <int D, int QC, bool SHARED = false>
 __device__ __forceinline__ float refine_pass(float2 (&hr)[D / 2], float2 (&hi)[D / 2], float *qre, float *qim,
                                              float *hre, float *him, const float2 *rpk, const float *gsrc, int j,
                                              bool again, bool apply) {
@@ -486,10 +488,11 @@ __device__ __forceinline__ float refine_pass(float2 (&hr)[D / 2], float2 (&hi)[D
     // first chain's row, in bounds, whose result is not used)
     const float2 mjj = sum_products_exact<D>(hr, hi, gsrc + 2 * d + j * D, gsrc + 3 * d + j * D, 192.0f, 0.0f);
     __syncwarp();
+    static_assert(!SHARED || D <= 16, "the rolled tail solves in place: one lane per row");
     if constexpr (D >= 32)
         return refine_tail_rolled<D, QC>(qre, qim, hre, him, rpk, j, mjj, apply);
     else
-        return refine_tail<D, QC>(qre, qim, hre, him, rpk, j, mjj, apply);
+        return refine_tail<D, QC, SHARED>(qre, qim, hre, him, rpk, j, mjj, apply);
 }
 
 // refine_pass's first pass where two groups of D lanes share a chain: the groups take the entries of
@@ -512,20 +515,20 @@ __device__ __forceinline__ float refine_pass_split(const float2 (&hr)[D / 2], co
     }
     const float2 mjj = sum_products_exact<D>(hr, hi, gsrc + 2 * d + j * D, gsrc + 3 * d + j * D, 192.0f, 0.0f);
     __syncwarp();
-    return refine_tail<D, QC, 2>(qre, qim, hre, him, rpk, j, mjj, true, grp);
+    return refine_tail<D, QC, true, 2>(qre, qim, hre, him, rpk, j, mjj, true, grp);
 }
 
 // The passes after the first, for the few chains whose first pass left |Y| above kRefineTol: out
 // of line, so that the common path keeps its registers.  `own`: this lane writes its column of U (where
-// several lanes repeat a chain's columns, one of them does).
-template <int D, int QC>
+// several lanes repeat a chain's columns (SHARED), one of them does).
+template <int D, int QC, bool SHARED>
 __device__ __noinline__ void refine_more(float *qre, float *qim, float *hre, float *him, const float2 *rpk,
                                          const float *gsrc, int j, float ymax, bool own) {
     float2 hr[D / 2], hi[D / 2];
 #pragma unroll 1
     for (int pass = 1; pass < kRefinePasses && __any_sync(0xffffffffu, ymax > kRefineTol); ++pass) {
         const bool need = ymax > kRefineTol;
-        const float next = refine_pass<D, QC>(hr, hi, qre, qim, hre, him, rpk, gsrc, j, true, need && own);
+        const float next = refine_pass<D, QC, SHARED>(hr, hi, qre, qim, hre, him, rpk, gsrc, j, true, need && own);
         ymax = need ? next : ymax;
     }
 }
