@@ -470,7 +470,8 @@ __global__ void __launch_bounds__(kWarp, kMinCtas) fused_small_kernel(const __gr
             v = part[0];
             if (NP > 1 && LPC < K) v += part[NP > 1 ? 1 : 0];
             if (NP > 2 && 2 * LPC < K) v += part[NP > 2 ? 2 : 0] + part[NP > 3 ? 3 : 0];
-            if (GRP > 1) v = __shfl_sync(0xffffffffu, v, 0, LPC);   // (a small tree's sum is in its own lanes)
+            // fewer settings than lanes: the tree's sum is in its own lanes only, and all of the chain's need it
+            if (K < LPC) v = __shfl_sync(0xffffffffu, v, 0, LPC);   // (uniform)
         }
 
         // ---- accept, adaptation (accept_kernel, phase 1) ----
