@@ -1138,6 +1138,38 @@ qst_status build_step_graph(qst_handle *h) {
     return QST_OK;
 }
 
+// The launches of qst_run_chains between the fork and the join of `forked` branches: the problems `multi`
+// on those, `num_steps` steps of the others (`steps`: there are some) on the handle's stream.
+qst_status enqueue_run(qst_handle *h, const std::vector<HostProblem *> &multi, int64_t num_steps, bool graph,
+                       bool steps, int forked) {
+    for (size_t i = 0; i < multi.size(); ++i) {
+        qst_status st = enqueue_multi(h, *multi[i], num_steps, forked ? h->branch[i % forked] : h->stream);
+        if (st != QST_OK) return st;
+    }
+    for (int64_t s = 0; s < num_steps; ++s) {
+        const int64_t j = h->steps_done + 1;
+        const bool kept = (j % h->cfg.thin == 0) && (j > h->cfg.burn_in);   // as the accept kernel decides it
+        if (graph) {
+            QST_CUDA(cudaGraphLaunch(h->graph_exec, h->stream), "launch step graph");
+            h->launches += h->graph_kernels;
+        } else if (steps) {
+            qst_status st = enqueue_step(h, false, !h->prof);
+            if (st != QST_OK) return st;
+        }
+        h->steps_done = j;
+        if (kept) h->kept += 1;
+    }
+    return QST_OK;
+}
+
+qst_status join_branches(qst_handle *h, int forked) {
+    for (int b = 0; b < forked; ++b) {
+        QST_CUDA(cudaEventRecord(h->join_ev[b], h->branch[b]), "join");
+        QST_CUDA(cudaStreamWaitEvent(h->stream, h->join_ev[b], 0), "join wait");
+    }
+    return QST_OK;
+}
+
 }  // namespace
 
 qst_status qst_run_chains(qst_handle *h, int64_t num_steps) {
@@ -1157,36 +1189,19 @@ qst_status qst_run_chains(qst_handle *h, int64_t num_steps) {
         if (st != QST_OK) return st;
     }
     int forked = 0;
-    if (!multi.empty()) {
-        qst_status st = QST_OK;
-        if (steps || multi.size() > 1) {   // on their own branches, beside the other problems
-            st = create_branches(h);
-            if (st != QST_OK) return st;
-            forked = (int)std::min<size_t>(multi.size(), qst_handle::kBranches);
-            QST_CUDA(cudaEventRecord(h->fork_ev, h->stream), "fork");
-            for (int b = 0; b < forked; ++b) QST_CUDA(cudaStreamWaitEvent(h->branch[b], h->fork_ev, 0), "branch wait");
-        }
-        for (size_t i = 0; i < multi.size() && st == QST_OK; ++i)
-            st = enqueue_multi(h, *multi[i], num_steps, forked ? h->branch[i % forked] : h->stream);
+    if (!multi.empty() && (steps || multi.size() > 1)) {   // on their own branches, beside the other problems
+        qst_status st = create_branches(h);
         if (st != QST_OK) return st;
+        forked = (int)std::min<size_t>(multi.size(), qst_handle::kBranches);
+        QST_CUDA(cudaEventRecord(h->fork_ev, h->stream), "fork");
+        for (int b = 0; b < forked; ++b) QST_CUDA(cudaStreamWaitEvent(h->branch[b], h->fork_ev, 0), "branch wait");
     }
-    for (int64_t s = 0; s < num_steps; ++s) {
-        const int64_t j = h->steps_done + 1;
-        const bool kept = (j % h->cfg.thin == 0) && (j > h->cfg.burn_in);   // as the accept kernel decides it
-        if (graph) {
-            QST_CUDA(cudaGraphLaunch(h->graph_exec, h->stream), "launch step graph");
-            h->launches += h->graph_kernels;
-        } else if (steps) {
-            qst_status st = enqueue_step(h, false, !h->prof);
-            if (st != QST_OK) return st;
-        }
-        h->steps_done = j;
-        if (kept) h->kept += 1;
-    }
-    for (int b = 0; b < forked; ++b) {
-        QST_CUDA(cudaEventRecord(h->join_ev[b], h->branch[b]), "join");
-        QST_CUDA(cudaStreamWaitEvent(h->stream, h->join_ev[b], 0), "join wait");
-    }
+    qst_status st = enqueue_run(h, multi, num_steps, graph, steps, forked);
+    // the branches join whether or not everything was launched: what follows on the handle's stream (or
+    // its destruction) must not overtake what was
+    const qst_status joined = join_branches(h, forked);
+    if (st == QST_OK) st = joined;
+    if (st != QST_OK) return st;
     if (multi.empty()) return QST_OK;
     return launch(h, QST_KERNEL_ACCEPT, "advance steps", [&] {   // (their launches have all read the counters)
         return launch_advance_steps(h->d_step, (int)h->plan.probs.size(), (uint32_t)num_steps, h->stream);
