@@ -539,8 +539,9 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
             acf_part = std::max(acf_part, sizeof(double) * (size_t)hp.v.n_diag * acf_slabs(hp.v.d) * (cfg->acf_lmax + 1));
     plan.acf_part_off = take(acf_part);
     plan.clear_bytes = off;   // what follows is written before it is read
-    for (auto &hp : plan.probs)
-        hp.hist_off = take(sizeof(float) * (size_t)fused_kept_steps(hp.v) * hp.v.R * hp.v.d);
+    for (auto &hp : plan.probs)   // a history only where some form of the problem runs many steps per launch
+        if (fused_possible(hp.v, hp.can_pauli))
+            hp.hist_off = take(sizeof(float) * (size_t)fused_kept_steps(hp.v) * hp.v.R * hp.v.d);
     plan.bytes = off;
     return QST_OK;
 }

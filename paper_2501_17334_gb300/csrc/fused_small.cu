@@ -650,18 +650,16 @@ cudaError_t launch_steps_d(const FusedArgs &a, cudaStream_t s) {
 // 38 us here against 58 us in per-step kernels in the FP32 form, and 32 us against 33 us in the Pauli
 // form, where the chip is full either way; 262144 one-qubit chains take 36 against 87 us.
 constexpr int64_t kFusedMaxState = 1 << 20;
-bool fused_supported(const ProblemView &p) {
-    if (p.D > 4 || (p.tc_kind != TC_NONE && !p.pauli)) return false;
+bool fused_possible(const ProblemView &p, bool may_be_pauli) {
+    if (p.D > 4 || p.R * p.d > kFusedMaxState) return false;
     if (p.qr_passes != 0 && p.qr_passes != 3) return false;
-    if (p.R * p.d > kFusedMaxState) return false;
-    if (p.pauli) return true;
-    return p.ngroups == 1 && p.KD / p.D <= kSettingSlots * p.D && p.KD <= 128;
+    if (p.pauli || may_be_pauli) return true;
+    return p.tc_kind == TC_NONE && p.KD / p.D <= kSettingSlots * p.D && p.KD <= 128;
 }
+bool fused_supported(const ProblemView &p) { return fused_possible(p, false) && (p.pauli || p.ngroups == 1); }
 
-// Kept steps one launch may cover: a history of at most 16 MB, and 512 of them.  0 where no choice
-// of the projection's form makes the problem one of this kernel's.
+// Kept steps one launch may cover: a history of at most 16 MB, and 512 of them.
 int fused_kept_steps(const ProblemView &p) {
-    if (p.D > 4 || p.R * p.d > kFusedMaxState) return 0;
     const int64_t row = p.R * p.d * (int64_t)sizeof(float);
     return (int)std::min<int64_t>(512, (16ll << 20) / row);
 }

@@ -233,6 +233,8 @@ cudaError_t launch_inject_nan(const ProblemView &p, int64_t chain, cudaStream_t 
 // launch covers nsteps steps with at most fused_kept_steps(p) kept ones, whose states go to `hist`
 // ([kept step][R][d] floats) for launch_fused_pool.
 bool fused_supported(const ProblemView &p);
+// the same before the projection's form is chosen (may_be_pauli: the structured form is one of the choices)
+bool fused_possible(const ProblemView &p, bool may_be_pauli);
 int fused_kept_steps(const ProblemView &p);
 cudaError_t launch_fused_steps(const ProblemView &p, const SamplerParams &sp, const StepState *base, uint32_t off,
                                int nsteps, int thin, int64_t burn_in, float *hist, cudaStream_t s);

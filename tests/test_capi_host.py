@@ -216,3 +216,23 @@ def test_huge_povm_count_is_rejected_before_any_product_wraps(qst):
         st = lib.qst_loglik_noalloc(4, k, None, counts.ctypes.data, None, 1, None, None)
         assert st == 1, (k, st)
     assert lib.qst_loglik_noalloc(4, 81, None, counts.ctypes.data, None, 1, None, None) == 1   # NULL P
+
+
+def test_history_only_where_steps_share_a_launch(qst):
+    """The workspace holds kept states of a many-step launch (16 MB at the largest such problem, 65536
+    two-qubit chains) only if one of the problem's forms has such launches; one chain more never has."""
+    def history(prob, **cfg):
+        sizes = []
+        for chains in (65536, 65537):
+            prob.num_chains = chains
+            sizes.append(qst.workspace_size([prob], qst.default_config(diag_chains=0, **cfg)))
+        return (sizes[0] - sizes[1] + (1 << 19)) >> 20   # in MB (a chain takes about 2 KB)
+    pauli = W.config_problem(2, num_chains=1)
+    assert history(pauli) == history(pauli, precision=qst.PREC_PAULI) == history(pauli, precision=qst.PREC_AUTO) == 16
+    assert history(pauli, prior=qst.PRIOR_HS, qr_passes=1) == 16
+    assert history(W.random_basis_problem(2, 16)) == 16
+    for cfg in (dict(precision=qst.PREC_BF16X3), dict(precision=qst.PREC_TF32), dict(precision=qst.PREC_TF32X2),
+                dict(qr_passes=1), dict(qr_passes=2, precision=qst.PREC_PAULI)):
+        assert history(pauli, **cfg) == 0, cfg
+    assert history(W.random_basis_problem(2, 17)) == 0          # more settings than a launch's lanes take
+    assert history(W.dyadic_basis_problem(2), precision=qst.PREC_AUTO) == 0   # tensor cores only
