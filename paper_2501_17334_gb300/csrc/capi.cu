@@ -497,7 +497,7 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
         Layout &L = hp.off;
         const int64_t R = v.R;
         L.P32 = take(sizeof(float) * hp.P32.size());
-        const bool lists = !tc && !hp.P32.empty() && fp32_lists(v);   // the FP32 form may run
+        const bool lists = !tc && !pauli && fp32_lists(v);   // the FP32 form runs
         L.sp_val = take(lists ? sizeof(float) * fp32_list_values(v) : 0);
         L.sp_code = take(lists ? sizeof(uint32_t) * fp32_list_codes(v) : 0);
         L.sp_len = take(lists ? sizeof(uint16_t) * fp32_list_lengths(v) : 0);
