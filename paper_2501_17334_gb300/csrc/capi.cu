@@ -93,7 +93,7 @@ bool bf16_exact(double v) {
 struct Layout {
     size_t P32, sp_val, sp_code, sp_len, Ptc, cnt, invf, ptot, colw, pauli_wq, pauli_wc, pauli_perm, y, cur, rho_cur, rho_prop, rho_split, trace_prop, logl_cur, logl_part, beta, coef,
         acc_win,
-        acc_total, pool, traj, trace_acc, trace_logl, red, acf, logl_eval, end;
+        acc_total, pool, traj, trace_acc, trace_logl, red, acf, logl_eval, end, list_part;
 };
 
 struct HostProblem {
@@ -447,6 +447,7 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
             v.pauli = pauli ? 1 : 0;
         }
         // column groups: a fixed rule, and the candidates the autotuner may time instead
+        int saved_slots = 0;   // partial sums per chain in a checkpoint, where not as many as are kept
         if (tc) {
             hp.tc_groups_rule = tc_ngroups(v, v.R);
             const int ntiles = v.KD_tc / tc_column_tile(v.D, v.KD);
@@ -465,10 +466,11 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
             hp.group_choices = hp.tc_group_choices;
         } else {
             v.ngroups = fp32_ngroups(v, v.R);
+            const int nt = v.KD_pad / 128;
             if (fp32_lists(v)) {   // an even share for every SM: nothing to tune
                 hp.group_choices = {v.ngroups};
+                saved_slots = nt;
             } else {
-                const int nt = v.KD_pad / 128;
                 for (int g = 1; g < nt; g *= 2) hp.group_choices.push_back(g);
                 hp.group_choices.push_back(nt);
             }
@@ -476,6 +478,8 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
         hp.part_slots = v.ngroups;
         for (int g : hp.group_choices) hp.part_slots = std::max(hp.part_slots, g);
         for (int g : hp.tc_group_choices) hp.part_slots = std::max(hp.part_slots, g);
+        if (saved_slots > 0) hp.part_slots = std::max(hp.part_slots, saved_slots);
+        else saved_slots = hp.part_slots;
         // the passes this problem's proposal kernel runs: 0, no QR (W = G); the refinement (3) at
         // D <= 16, and at D = 32 only when 4 is asked for; D = 64 has the first-order form (2)
         v.qr_passes = cfg->prior == QST_PRIOR_HS ? 0 : cfg->qr_passes;
@@ -517,7 +521,7 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
         L.rho_split = take(tc ? (size_t)tc_elem_bytes(kind) * tc_splits(kind) * R * v.d_pad : 0);
         L.trace_prop = take(sizeof(double) * R);
         L.logl_cur = take(sizeof(double) * R);
-        L.logl_part = take(sizeof(double) * hp.part_slots * R);
+        L.logl_part = take(sizeof(double) * saved_slots * R);
         L.beta = take(sizeof(double) * R);
         L.coef = take(sizeof(float2) * R);
         L.acc_win = take(sizeof(int32_t) * R);
@@ -530,6 +534,9 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
         L.acf = take(sizeof(double) * (size_t)std::max(v.n_diag, 1) * (cfg->acf_lmax + 1));
         L.logl_eval = take(sizeof(double) * R);
         L.end = off;
+        // The list projection's partial sums where it has more of them: beside the saved region, whose size
+        // (one slot per column tile of P, as the tiled FP32 kernel needs) is a checkpoint's format.
+        L.list_part = hp.part_slots > saved_slots ? take(sizeof(double) * hp.part_slots * R) : L.logl_part;
     }
     plan.status_off = take(256);
     plan.step_off = take(sizeof(StepState) * plan.probs.size());
@@ -658,7 +665,7 @@ qst_status bind_problem(qst_handle *h, HostProblem &hp) {
     v.rho_split = b + L.rho_split;
     v.trace_prop = reinterpret_cast<double *>(b + L.trace_prop);
     v.logl_cur = reinterpret_cast<double *>(b + L.logl_cur);
-    v.logl_part = reinterpret_cast<double *>(b + L.logl_part);
+    v.logl_part = reinterpret_cast<double *>(b + L.list_part);
     v.beta = reinterpret_cast<double *>(b + L.beta);
     v.coef = reinterpret_cast<float2 *>(b + L.coef);
     v.acc_win = reinterpret_cast<int32_t *>(b + L.acc_win);
