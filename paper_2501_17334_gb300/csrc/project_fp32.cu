@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(256) project_fp32_small_kernel(ProjectArgs a, 
 // length of their lists, are laid end to end by cost (rows plus kSpEpilogue for the logarithms) and
 // cut into equal pieces, one per CTA, so that all SMs are busy whatever the number of chains; a tile
 // that several CTAs share has one partial sum per CTA.
-// 10007 four-qubit chains with p written take 103 us, 65536 without 453 us, against 330 and 1740 us by
+// 10007 four-qubit chains with p written take 103 us, 65536 without 465 us, against 330 and 1740 us by
 // the tiled kernel (an FMA-bound time would be 32 and 210 us: with 255 registers two warps share a
 // scheduler, and a row's 128-bit loads keep the shared-memory pipe half busy).
 constexpr int kSpStages = 3;
@@ -414,6 +414,15 @@ __device__ __forceinline__ void st_global_8(float *dst, const float (&v)[8]) {
                  "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
                  : "memory");
 }
+
+// sum + rest += c v: the product's part on the grid of `sum` (whose exponent no add changes), and the rest of
+// it, which the second FMA forms exactly
+__device__ __forceinline__ void add_product(float2 &sum, float2 &rest, float2 c, float2 v) {
+    const float2 n = fma2(c, v, sum);
+    rest = add2(rest, fma2(c, v, sub2(sum, n)));
+    sum = n;
+}
+__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
 
 template <int D, int C, bool POISSON, bool P_OUT>
 __global__ void __launch_bounds__(SparseShape<D, C>::threads, 1) project_fp32_sparse_kernel(SparseArgs a) {
@@ -686,11 +695,26 @@ __global__ void __launch_bounds__(SparseShape<D, C>::threads, 1) project_fp32_sp
                     if (!has_second(k)) add_setting(tot_hi[i], tot_lo[i], run[i], run_c[i], -run_small[i]);
                 }
             } else if (pk > 0.0f) {
-                float2 sh[C], sl[C], dev[C], comp[C];
+                // The setting's sum starts at 1.5 2^k, with 2^(k-1) above any sum of its terms (counts below
+                // 2^(e+1) in all, |log| < 2^7, k = e + 9), so it stays on one grid and add_product loses
+                // nothing.  (A Kahan sum from zero took as many instructions, rounded every product and lost part
+                // of an add's error whenever a term was larger than the sum so far.  rms error of log L on
+                // the stored rho, relative, over 60000 four-qubit Pauli states: the tiled kernel's sums
+                // 8.40e-10, Kahan sums from zero 8.44e-10, these 7.33e-10.
+                // Where the compiler schedules them worst, 65536 chains without p, they cost 453 -> 465 us.)
+                float total = pk;
+                if constexpr (POISSON) {   // the counts may exceed mu
+                    total = 0.0f;
+#pragma unroll
+                    for (int l = 0; l < D; ++l) total += wts[2 * D + l];
+                }
+                const float base = __int_as_float((__float_as_int(total) & 0x7f800000) + (9 << 23) + 0x400000);
+                float2 sh[C], sl[C], dev[C], rest[C];
                 int xmin[C];
 #pragma unroll
                 for (int i = 0; i < C; ++i) {
-                    sh[i] = sl[i] = dev[i] = comp[i] = splat2(0.0f);
+                    sh[i] = sl[i] = rest[i] = splat2(0.0f);
+                    dev[i] = splat2(base);
                     xmin[i] = 0x7fffffff;
                 }
 #pragma unroll
@@ -705,22 +729,23 @@ __global__ void __launch_bounds__(SparseShape<D, C>::threads, 1) project_fp32_sp
                         sl[i] = add2(sl[i], sub2(q, h));
                         const float2 x = fma2(q, make_float2(w.x, w.y), make_float2(w.z, w.w));
                         xmin[i] = min(xmin[i], min(__float_as_int(x.x), __float_as_int(x.y)));
-                        kahan_fma2(dev[i], comp[i], cn, log_poly2(x));
+                        add_product(dev[i], rest[i], cn, log_poly2(x));
                     }
                 }
 #pragma unroll
                 for (int i = 0; i < C; ++i) {
+                    dev[i] = sub2(dev[i], splat2(base));   // (exact)
                     const float s_hi = sh[i].x + sh[i].y, s_lo = sl[i].x + sl[i].y;
                     if constexpr (POISSON) {
                         float ph, pl;
                         poisson_setting(pk, s_hi, s_lo, t_hi[i], t_lo[i], ph, pl);
-                        add_setting_pair(tot_hi[i], tot_lo[i], dev[i], comp[i], ph, pl);
+                        add_setting_pair(tot_hi[i], tot_lo[i], dev[i], neg2(rest[i]), ph, pl);
                     } else {
                         const float rel = ((s_hi - t_hi[i]) + (s_lo - t_lo[i])) * inv_t[i];
                         const float l1p = fabsf(rel) < 0x1p-10f
                                               ? rel * __fmaf_rn(rel, __fmaf_rn(rel, 0.33333334f, -0.5f), 1.0f)
                                               : log1pf(rel);
-                        add_setting(tot_hi[i], tot_lo[i], dev[i], comp[i], pk * l1p);
+                        add_setting(tot_hi[i], tot_lo[i], dev[i], neg2(rest[i]), pk * l1p);
                     }
                     dead[i] |= xmin[i] < 0x00800000;
                 }
