@@ -291,6 +291,22 @@ void pauli_povms(int Q, std::vector<double> &re, std::vector<double> &im) {
                 }
 }
 
+// The rows of P each setting's list will hold (those where one of its elements is not zero, or one)
+void count_list_rows(HostProblem &hp) {
+    ProblemView &v = hp.v;
+    v.sp_rows = 0;
+    v.sp_most = 0;
+    for (int k = 0; k < hp.K; ++k) {
+        int n = 0;
+        for (int r = 0; r < v.d; ++r) {
+            const float *row = hp.P32.data() + (size_t)r * v.KD_pad + k * v.D;
+            n += std::any_of(row, row + v.D, [](float x) { return !(x == 0.0f); }) ? 1 : 0;
+        }
+        v.sp_rows += std::max(n, 1);
+        v.sp_most = std::max(v.sp_most, std::max(n, 1));
+    }
+}
+
 qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_sampler_cfg *cfg, Plan &plan) {
     if (!probs_in || n < 1) return fail(QST_ERR_INVALID_ARG, "need at least one problem");
     qst_status st = validate_cfg(cfg);
@@ -465,11 +481,12 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
             v.ngroups = hp.tc_groups_rule;
             hp.group_choices = hp.tc_group_choices;
         } else {
+            if (fp32_lists(v)) count_list_rows(hp);
             v.ngroups = fp32_ngroups(v, v.R);
             const int nt = v.KD_pad / 128;
-            if (fp32_lists(v)) {   // an even share for every SM: nothing to tune
+            if (fp32_lists(v)) saved_slots = nt;
+            if (fp32_list_form(v, v.R)) {   // an even share for every SM: nothing to tune
                 hp.group_choices = {v.ngroups};
-                saved_slots = nt;
             } else {
                 for (int g = 1; g < nt; g *= 2) hp.group_choices.push_back(g);
                 hp.group_choices.push_back(nt);
@@ -1494,10 +1511,10 @@ qst_status qst_evaluate(qst_handle *h, int32_t problem, const float *x, int64_t 
         return launch_propose(v, MODE_EVAL, 0u, nullptr, x, n, uses_tc(v), rho, h->d_status, h->stream);
     });
     if (st != QST_OK) return st;
-    // a batch smaller than the chains: the FP32 form's CTAs may share its tiles more finely (as far as
-    // the partial sums' buffer goes)
+    // a batch smaller than the chains: the list kernel's CTAs may share its tiles more finely (as far as
+    // the partial sums' buffer goes), and the kernel may be the other one
     const int groups = v.ngroups;
-    if (hp->lists)
+    if (hp->lists && (fp32_list_form(v, n) || fp32_list_form(v, v.R)))
         v.ngroups = (int)std::max<int64_t>(1, std::min<int64_t>(fp32_ngroups(v, n), (int64_t)hp->part_slots * v.R / n));
     st = enqueue_projection(h, *hp, n, p);
     if (st == QST_OK && logl)

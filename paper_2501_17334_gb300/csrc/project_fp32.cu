@@ -866,12 +866,29 @@ cudaError_t launch_fp32_lists(const ProblemView &p, const float *P, int ld, floa
 }
 
 namespace {
+constexpr int kSms = 152;
+int sparse_units(const ProblemView &p) {   // of a tile: settings, at D = 8 pairs of them
+    const int K = p.KD / p.D;
+    return p.D == 8 ? K / 16 * 8 + std::min(8, K % 16) : K;
+}
+// rows of P over all settings' lists, each with kSpEpilogue for its logarithms (a Pauli problem's number
+// where the lists are not known on the host)
+int64_t sparse_cost(const ProblemView &p) {
+    const int64_t K = p.KD / p.D;
+    return (p.sp_rows > 0 ? p.sp_rows : (p.D == 16 ? 70 : 23) * K) + kSpEpilogue * K;
+}
 // Chains per lane: four (the row's P entries serve 128 chains), or one (shorter settings, more of them)
-// while there are few settings per warp.  us at four / one chains per lane, Pauli settings with p
-// written: four qubits 1 row 27 / 17, 1000 rows 43 / 31, 4096 rows 68 / 59, 6000 rows 77 / 80, 10007
-// rows 103 / 119; three qubits 1000 rows 20 / 14, 6000 rows 24 / 23, 10007 rows 25 / 29.
+// while there is little work per warp.  us at four / one chains per lane with p written, Pauli settings:
+// four qubits 1 row 27 / 17, 1000 rows 43 / 31, 4096 rows 68 / 59, 6000 rows 77 / 80, 10007 rows 103 / 119;
+// three qubits 1000 rows 20 / 14, 6000 rows 24 / 23, 10007 rows 25 / 29.  So the line at four qubits lies
+// at 40 tiles of 128 chains, or as many listed rows where the lists are longer (81 bases without zeros: 2000
+// rows 72 / 84, 3000 rows 90 / 109).  A few settings take four as well while every CTA then has one, but
+// two or more with one (a setting without zeros, 16384 rows: 33 / 63; 16 of them, 1000 rows: 33 / 35).
 int sparse_c(const ProblemView &p, int64_t rows) {
-    return (rows + 127) / 128 * (p.KD / p.D) >= (p.D == 16 ? 3200 : 1600) ? 4 : 1;
+    const int64_t K = p.KD / p.D, tiles = (rows + 127) / 128;
+    if (p.D == 8) return tiles * K >= 1600 ? 4 : 1;
+    if (tiles * sparse_cost(p) >= 300000) return 4;
+    return K <= 16 && tiles * K <= kSms && (rows + 31) / 32 * K > 2 * kSms ? 4 : 1;
 }
 // CTAs of the sparse kernel: one per SM (fewer only where there are fewer settings); a tile's piece of
 // the costs then meets at most ceil(CTAs / tiles) + 1 of them
@@ -880,14 +897,43 @@ int64_t sparse_tiles(const ProblemView &p, int64_t rows) {
     return (rows + M - 1) / M;
 }
 int64_t sparse_ctas(const ProblemView &p, int64_t rows) {
-    const int64_t K = p.KD / p.D, units = p.D == 8 ? K / 16 * 8 + std::min<int64_t>(8, K % 16) : K;
-    return std::min<int64_t>(152, sparse_tiles(p, rows) * units);
+    return std::min<int64_t>(kSms, sparse_tiles(p, rows) * sparse_units(p));
 }
 int sparse_groups(int64_t tiles, int64_t ctas) { return (int)((ctas + tiles - 1) / tiles) + 1; }
 }  // namespace
 
+// Whether the list kernel is the faster one at this many rows.  The tiled kernel takes a wave of tiles of
+// 128 rows x 128 columns after the other; the list kernel an even share of the listed rows for every SM, but at
+// least a setting's list per warp, twice where a CTA's share spans two tiles, and the ordering of
+// many settings.  Lists without zeros save nothing, so around whole waves of tiles the tiled kernel wins.  us by
+// these estimates and measured, tiled / list: four qubits, 81 bases 1000 rows 56 / 58 (57 / 58), 1500 rows
+// 56 / 70 (56 / 66), 2000 rows 100 / 73 (99 / 68); 1000 bases 64 rows 56 / 101 (56 / 97), 1000 rows 318 / 282
+// (353 / 305); Pauli settings 1500 rows 56 / 29 (57 / 35); three qubits, 300 bases 1000 rows 33 / 35 (33 / 35), 1400
+// rows 51 / 38 (51 / 39).
+bool fp32_list_form(const ProblemView &p, int64_t rows) {
+    if (!fp32_lists(p)) return false;
+    if (p.sp_rows == 0) return true;   // the lists' lengths are not known on the host
+    const int64_t tiles = (rows + 127) / 128, K = p.KD / p.D, units = sparse_units(p), total = sparse_cost(p);
+    const double waves = (double)((tiles * (p.KD_pad / BN) + kSms - 1) / kSms);
+    const double cost = (double)total / kSms;   // per tile and SM
+    const double one = (p.sp_most + kSpEpilogue) * (units < K ? 2.0 : 1.0);
+    // the CTAs' even shares end inside tiles, unless they happen to divide them
+    auto spans = [&](int64_t t) { return t > 1 && t * units > kSms && (kSms % t != 0 || t * total % kSms != 0); };
+    double list;
+    if (p.D == 8) {
+        list = 9.0 + 0.05 * (tiles * cost / 8 + one * (spans(tiles) ? 1.58 : 1.0)) + 0.0244 * units * ((units + 255) / 256);
+    } else if (sparse_c(p, rows) == 4) {
+        list = 6.0 + 0.085 * (tiles * cost / 8 + one * (spans(tiles) ? 1.67 : 1.0)) + 0.02 * K * ((K + 255) / 256);
+    } else {
+        const int64_t t32 = (rows + 31) / 32;
+        const double more = !spans(t32) ? 1.0 : t32 >= 2 * kSms ? 0.35 : 1.35;
+        list = 3.0 + 0.079 * (t32 * cost / 16 * std::max(1.0, 12.0 / K) + one * more) + 0.025 * K * ((K + 511) / 512);
+    }
+    return list <= (p.D == 8 ? 14.0 + 18.7 * waves : 13.0 + 43.5 * waves);
+}
+
 int fp32_ngroups(const ProblemView &p, int64_t rows) {
-    if (fp32_lists(p)) return sparse_groups(sparse_tiles(p, rows), sparse_ctas(p, rows));
+    if (fp32_list_form(p, rows)) return sparse_groups(sparse_tiles(p, rows), sparse_ctas(p, rows));
     // enough CTAs to fill the machine: split the columns when there are few row tiles
     const int64_t mt = (rows + BM - 1) / BM;
     const int nt = p.KD_pad / BN;
@@ -980,7 +1026,7 @@ cudaError_t launch_project_fp32(const ProblemView &p, const float *A, int64_t ro
         }
         return cudaGetLastError();
     }
-    if (p.sp_val) {
+    if (p.sp_val && fp32_list_form(p, rows)) {
         SparseArgs b;
         b.A = A;
         b.val = p.sp_val;

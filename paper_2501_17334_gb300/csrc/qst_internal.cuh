@@ -158,7 +158,9 @@ struct ProblemView {
     const float *sp_val;         // FP32 form at D = 8, 16 (null otherwise): per setting the rows of P where any
                                  //                  of its elements is nonzero, [K][d][D],
     const uint32_t *sp_code;     //                  their row codes [K][d]
-    const uint16_t *sp_len;      //                  and the number of rows listed [K]
+    const uint16_t *sp_len;      //                  and the number of rows listed [K];
+    int64_t sp_rows;             //                  their sum and the most of one setting, where the host
+    int sp_most;                 //                  knows them (0 otherwise)
     const void *Ptc;             // [KD_tc][d_pad]   tensor-core B operand (row = projector, contiguous packed
                                  //                  index): bf16, or FP32 holding TF32 values
     const float *cnt;            // [max(KD_pad, KD_tc)] counts as float, 0 on padding
@@ -256,8 +258,10 @@ bool tc_supported(int kind, int D);      // the tensor-core kernels handle this 
 // test hook: one bounded mbarrier wait that nothing satisfies (sets STATUS_TIMEOUT after limit_ns)
 cudaError_t launch_wait_timeout_probe(uint32_t *status, uint64_t limit_ns, cudaStream_t s);
 int fp32_ngroups(const ProblemView &p, int64_t rows);
-// The FP32 form's lists of used rows per setting (project_fp32.cu): whether this size has them, the
+// The FP32 form's lists of used rows per setting (project_fp32.cu): whether a call of `rows` rows takes
+// the list kernel (else the tiled one), whether this size has them, the
 // floats, codes and lengths they take, and the kernel that makes them from P ([d][ld], device).
+bool fp32_list_form(const ProblemView &p, int64_t rows);
 bool fp32_lists(const ProblemView &p);
 size_t fp32_list_values(const ProblemView &p);
 size_t fp32_list_codes(const ProblemView &p);
