@@ -596,9 +596,12 @@ struct qst_handle {
     static constexpr int kBranches = 8;      // problems of a graph step run on up to 8 parallel branches
     cudaStream_t branch[kBranches] = {};
     cudaEvent_t fork_ev = nullptr, join_ev[kBranches] = {};
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t graph_exec = nullptr;
-    int64_t graph_kernels = 0;               // kernel launches one replay performs
+    struct StepGraph {
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        int64_t kernels = 0;                 // kernel launches one replay performs
+    };
+    StepGraph steps_graph, single_graph;     // a step of the problems that go step by step, and of all of them
     int64_t steps_done = 0;
     int64_t kept = 0;
     int64_t launches = 0;
@@ -1137,8 +1140,8 @@ qst_status create_branches(qst_handle *h) {
     return QST_OK;
 }
 
-// Captures enqueue_step once on the private capture stream and instantiates it.
-qst_status build_step_graph(qst_handle *h) {
+// Captures enqueue_step once on the private capture stream and instantiates it (`multi` as there).
+qst_status build_step_graph(qst_handle *h, bool multi, qst_handle::StepGraph &out) {
     const qst_status made = create_branches(h);
     if (made != QST_OK) return made;
     cudaStream_t user = h->stream;
@@ -1146,11 +1149,11 @@ qst_status build_step_graph(qst_handle *h) {
     h->stream = h->capture_stream;
     cudaError_t e = cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal);
     qst_status st = QST_OK;
-    if (e == cudaSuccess) st = enqueue_step(h, true, true);
+    if (e == cudaSuccess) st = enqueue_step(h, true, multi);
     cudaGraph_t g = nullptr;
     const cudaError_t e_end = (e == cudaSuccess) ? cudaStreamEndCapture(h->capture_stream, &g) : e;
     h->stream = user;
-    h->graph_kernels = h->launches - launches0;
+    out.kernels = h->launches - launches0;
     h->launches = launches0;
     if (e != cudaSuccess) return cuda_fail(e, "begin graph capture");
     if (st != QST_OK) {
@@ -1158,15 +1161,62 @@ qst_status build_step_graph(qst_handle *h) {
         return st;
     }
     if (e_end != cudaSuccess) return cuda_fail(e_end, "end graph capture");
-    h->graph = g;
-    QST_CUDA(cudaGraphInstantiate(&h->graph_exec, g, 0), "instantiate step graph");
+    out.graph = g;
+    QST_CUDA(cudaGraphInstantiate(&out.exec, g, 0), "instantiate step graph");
     return QST_OK;
 }
 
+// A step of one problem by itself, us, roughly (measured: 64 chains to a full chip); at one and two qubits the
+// part that does not grow with the chains.
+double step_us(const ProblemView &v) {
+    switch (v.D) {
+        case 2: return 15.0;
+        case 4: return 17.0;
+        case 8: return 23.0 + 1.7e-3 * v.R;
+        case 16: return 38.0 + 1.0e-2 * v.R;
+        case 32: return 50.0 + 4.3e-2 * v.R;
+        default: return 60.0 + 0.4 * v.R;
+    }
+}
+
+// Whether the problems `multi` of the handle take many-step launches in a call of num_steps steps, or go step by
+// step with the others.
+//   Alone, such a launch, its pooling and the counters take about 16 us beyond the steps: one step costs
+// 20 us instead of 16 (64 one-qubit chains), two 22 instead of 31.  (65536 two-qubit chains in the Pauli form
+// gain least: two steps 85 instead of 82, three 110 instead of 124.)  Several such problems fork to branches and
+// join: two steps of eight two-qubit problems 65 instead of 54, three 73 instead of 80.
+//   Beside problems that go step by step, a small one on a branch of its own in the step graph costs nothing,
+// while its launches are extra and their CTAs slow the others down: one of 4096 two-qubit chains beside 16384
+// three-qubit ones 51.6 us per step instead of 48.3, six mixed problems two steps 136 instead of 93.  There the
+// launches pay where the small problems lengthen the graph's branches (30 one-qubit problems and a four-qubit
+// one 38 us per step instead of 75) or are large and spare the chip work (65536 two-qubit chains in the FP32 form
+// beside three-qubit ones 60 instead of 76; in the Pauli form they spare none).
+bool multi_step_pays(const qst_handle *h, const std::vector<HostProblem *> &multi, int64_t num_steps) {
+    if (multi.size() == h->plan.probs.size()) {
+        const ProblemView &v = multi[0]->v;
+        const bool least = v.pauli && v.D == 4 && v.R * v.d > (1 << 19);
+        return num_steps >= (multi.size() > 1 || least ? 3 : 2);
+    }
+    double whole[qst_handle::kBranches] = {}, rest[qst_handle::kBranches] = {}, saved = 0.0;
+    int i = 0, r = 0;
+    for (const auto &hp : h->plan.probs) {   // (as enqueue_step deals them to the branches)
+        const double us = step_us(hp.v);
+        whole[i++ % qst_handle::kBranches] += us;
+        if (!fused_supported(hp.v))
+            rest[r++ % qst_handle::kBranches] += us;
+        else if (hp.v.D == 2 || !hp.v.pauli)
+            saved += (hp.v.D == 2 ? 40.0 : 20.0) * (double)(hp.v.R * hp.v.d) / (1 << 20);
+    }
+    const int nb = qst_handle::kBranches;
+    saved += *std::max_element(whole, whole + nb) - *std::max_element(rest, rest + nb);
+    return num_steps * saved > 30.0 + 4.0 * multi.size();
+}
+
 // The launches of qst_run_chains between the fork and the join of `forked` branches: the problems `multi`
-// on those, `num_steps` steps of the others (`steps`: there are some) on the handle's stream.
-qst_status enqueue_run(qst_handle *h, const std::vector<HostProblem *> &multi, int64_t num_steps, bool graph,
-                       bool steps, int forked) {
+// on those, `num_steps` steps of the others (`steps`: there are some) on the handle's stream, by `graph`
+// where it is not null.
+qst_status enqueue_run(qst_handle *h, const std::vector<HostProblem *> &multi, int64_t num_steps,
+                       const qst_handle::StepGraph *graph, bool steps, int forked) {
     for (size_t i = 0; i < multi.size(); ++i) {
         qst_status st = enqueue_multi(h, *multi[i], num_steps, forked ? h->branch[i % forked] : h->stream);
         if (st != QST_OK) return st;
@@ -1175,10 +1225,10 @@ qst_status enqueue_run(qst_handle *h, const std::vector<HostProblem *> &multi, i
         const int64_t j = h->steps_done + 1;
         const bool kept = (j % h->cfg.thin == 0) && (j > h->cfg.burn_in);   // as the accept kernel decides it
         if (graph) {
-            QST_CUDA(cudaGraphLaunch(h->graph_exec, h->stream), "launch step graph");
-            h->launches += h->graph_kernels;
+            QST_CUDA(cudaGraphLaunch(graph->exec, h->stream), "launch step graph");
+            h->launches += graph->kernels;
         } else if (steps) {
-            qst_status st = enqueue_step(h, false, !h->prof);
+            qst_status st = enqueue_step(h, false, !multi.empty());
             if (st != QST_OK) return st;
         }
         h->steps_done = j;
@@ -1202,16 +1252,22 @@ qst_status qst_run_chains(qst_handle *h, int64_t num_steps) {
     if (num_steps < 0) return fail(QST_ERR_INVALID_ARG, "num_steps must be >= 0");
     if (h->steps_done + num_steps > 0xffffffffLL) return fail(QST_ERR_INVALID_ARG, "step counter exceeds 32 bits");
     if (num_steps == 0) return QST_OK;
-    // problems that run many steps per launch (kernel timing takes the per-step kernels instead)
+    // problems that run many steps per launch (kernel timing takes the per-step kernels instead, and so do
+    // calls too short for such launches)
     std::vector<HostProblem *> multi;
     if (!h->prof)
         for (auto &hp : h->plan.probs)
             if (fused_supported(hp.v)) multi.push_back(&hp);
+    const bool single = !multi.empty() && !multi_step_pays(h, multi, num_steps);   // all step by step
+    if (single) multi.clear();
     const bool steps = multi.size() < h->plan.probs.size();   // some problems go step by step
-    const bool graph = h->cfg.use_graph && !h->prof && steps;
-    if (graph && !h->graph_exec) {
-        qst_status st = build_step_graph(h);
-        if (st != QST_OK) return st;
+    qst_handle::StepGraph *graph = nullptr;
+    if (h->cfg.use_graph && !h->prof && steps) {
+        graph = single ? &h->single_graph : &h->steps_graph;
+        if (!graph->exec) {
+            qst_status st = build_step_graph(h, !multi.empty(), *graph);
+            if (st != QST_OK) return st;
+        }
     }
     int forked = 0;
     if (!multi.empty() && (steps || multi.size() > 1)) {   // on their own branches, beside the other problems
@@ -1403,8 +1459,10 @@ void qst_destroy(qst_handle *h) {
         cudaEventDestroy(ev.a);
         cudaEventDestroy(ev.b);
     }
-    if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
-    if (h->graph) cudaGraphDestroy(h->graph);
+    for (auto *g : {&h->steps_graph, &h->single_graph}) {
+        if (g->exec) cudaGraphExecDestroy(g->exec);
+        if (g->graph) cudaGraphDestroy(g->graph);
+    }
     if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
     for (int b = 0; b < qst_handle::kBranches; ++b) {
         if (h->branch[b]) cudaStreamDestroy(h->branch[b]);
