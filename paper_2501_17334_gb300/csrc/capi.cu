@@ -1092,6 +1092,14 @@ qst_status enqueue_step(qst_handle *h, bool branches, bool multi) {
     }
     const int nb = np < qst_handle::kBranches ? np : qst_handle::kBranches;
     cudaStream_t origin = h->stream;
+    // From three branches on they leave one node: a graph that starts with several kernels takes longer to
+    // start than one and its successors (us per step with / without it: six mixed problems 50.8 / 53.6, ten
+    // 50.1 / 53.1, 20000 one- and two-qubit and 500 five-qubit chains 61.7 / 68.8; two branches 26.2 / 25.0).
+    // Not beside many-step launches, which fill the chip anyway (thirteen problems 95 / 90).
+    if (nb > 2 && !multi) {
+        st = launch(h, QST_KERNEL_ACCEPT, "fork", [&] { return launch_fork(origin); });
+        if (st != QST_OK) return st;
+    }
     QST_CUDA(cudaEventRecord(h->fork_ev, origin), "fork");
     for (int b = 0; b < nb; ++b) QST_CUDA(cudaStreamWaitEvent(h->branch[b], h->fork_ev, 0), "branch wait");
     for (int i = 0; i < np && st == QST_OK; ++i) {
@@ -1204,8 +1212,9 @@ bool multi_step_pays(const qst_handle *h, const std::vector<HostProblem *> &mult
         whole[i++ % qst_handle::kBranches] += us;
         if (!fused_supported(hp.v))
             rest[r++ % qst_handle::kBranches] += us;
-        else if (hp.v.D == 2 || !hp.v.pauli)
-            saved += (hp.v.D == 2 ? 40.0 : 20.0) * (double)(hp.v.R * hp.v.d) / (1 << 20);
+        else   // (large ones; and FP32 projections of any size, whose kernels get in the others' way)
+            saved += (hp.v.D == 2 ? 40.0 : hp.v.pauli ? 0.0 : 20.0) * (double)(hp.v.R * hp.v.d) / (1 << 20) +
+                     (hp.v.pauli ? 0.0 : 1.2);
     }
     const int nb = qst_handle::kBranches;
     saved += *std::max_element(whole, whole + nb) - *std::max_element(rest, rest + nb);

@@ -606,6 +606,8 @@ __global__ void __launch_bounds__(kAdvanceThreads) advance_steps_kernel(StepStat
     }
 }
 
+__global__ void fork_kernel() {}
+
 template <int D, int PASSES, int LPC, bool PAULI, bool POISSON>
 cudaError_t launch_steps_w(const FusedArgs &a, cudaStream_t s) {
     using F = FusedShape<D, PASSES, LPC>;
@@ -685,6 +687,11 @@ cudaError_t launch_fused_pool(const ProblemView &p, const StepState *base, uint3
         fused_pool_kernel<2><<<p.n_slots, kPoolThreads, 0, s>>>(p, base, off, nsteps, thin, burn_in, hist);
     else
         fused_pool_kernel<4><<<p.n_slots, kPoolThreads, 0, s>>>(p, base, off, nsteps, thin, burn_in, hist);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fork(cudaStream_t s) {
+    fork_kernel<<<1, 1, 0, s>>>();
     return cudaGetLastError();
 }
 

@@ -242,6 +242,7 @@ cudaError_t launch_fused_steps(const ProblemView &p, const SamplerParams &sp, co
                                int nsteps, int thin, int64_t burn_in, float *hist, cudaStream_t s);
 cudaError_t launch_fused_pool(const ProblemView &p, const StepState *base, uint32_t off, int nsteps, int thin,
                               int64_t burn_in, const float *hist, cudaStream_t s);
+cudaError_t launch_fork(cudaStream_t s);   // a kernel that does nothing: the node a step graph's branches leave
 // n steps at once for those of the `count` problems that run many steps per launch
 cudaError_t launch_advance_steps(StepState *st, int count, uint32_t n, cudaStream_t s);
 
