@@ -1095,11 +1095,9 @@ qst_status enqueue_step(qst_handle *h, bool branches, bool multi) {
     // From three branches on they leave one node: a graph that starts with several kernels takes longer to
     // start than one and its successors (us per step with / without it: six mixed problems 50.8 / 53.6, ten
     // 50.1 / 53.1, 20000 one- and two-qubit and 500 five-qubit chains 61.7 / 68.8; two branches 26.2 / 25.0).
-    // Not beside many-step launches, which fill the chip anyway (thirteen problems 95 / 90).
-    if (nb > 2 && !multi) {
-        st = launch(h, QST_KERNEL_ACCEPT, "fork", [&] { return launch_fork(origin); });
-        if (st != QST_OK) return st;
-    }
+    // Not beside many-step launches, which fill the chip anyway (thirteen problems 95 / 90).  The node does
+    // nothing and is not among the launches counted, which are those of plain launches.
+    if (nb > 2 && !multi) QST_CUDA(launch_fork(origin), "fork");
     QST_CUDA(cudaEventRecord(h->fork_ev, origin), "fork");
     for (int b = 0; b < nb; ++b) QST_CUDA(cudaStreamWaitEvent(h->branch[b], h->fork_ev, 0), "branch wait");
     for (int i = 0; i < np && st == QST_OK; ++i) {

@@ -36,8 +36,8 @@ def test_calls_of_any_length(qst, cuda_ok, graph, sizes):
     ([(1, 500), (2, 500), (3, 500), (4, 500)], 10, False), ([(1, 17)] * 20 + [(3, 40)], 3, False),
     ([(1, 17)] * 20 + [(3, 40)], 12, True), ([(1, 65536), (3, 40)], 8, True)])
 def test_which_launches(qst, cuda_ok, sizes, steps, multi):
-    """Three kernels a problem and step and one where three or more branches leave, or two a problem (steps,
-    pooling) and one for the counters; the same chains as with kernel timing, which takes the per-step kernels."""
+    """Three kernels a problem and step, or two a problem (steps, pooling) and one for the counters; the
+    same chains as with kernel timing, which takes the per-step kernels."""
     probs = [W.config_problem(q, num_chains=R) for q, R in sizes]
     kw = dict(precision=qst.PREC_PAULI, diag_chains=0, thin=2)
     with qst.Sampler(probs, **kw) as s, qst.Sampler(probs, **kw) as plain:
@@ -45,7 +45,7 @@ def test_which_launches(qst, cuda_ok, sizes, steps, multi):
         before = s.launch_count()
         s.run_chains(steps)
         small = sum(q <= 2 for q, _ in sizes)
-        want = small * 2 + 1 + 3 * steps * (len(sizes) - small) if multi else (3 * len(sizes) + (len(sizes) > 2)) * steps
+        want = small * 2 + 1 + 3 * steps * (len(sizes) - small) if multi else 3 * steps * len(sizes)
         assert s.launch_count() - before == want
         s.run_chains(3)
         plain.run_chains(steps + 3)
