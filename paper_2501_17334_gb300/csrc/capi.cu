@@ -555,6 +555,10 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
         // (one slot per column tile of P, as the tiled FP32 kernel needs) is a checkpoint's format.
         L.list_part = hp.part_slots > saved_slots ? take(sizeof(double) * hp.part_slots * R) : L.logl_part;
     }
+    int64_t large = 0;
+    for (const auto &hp : plan.probs) large += hp.v.D >= 8 ? hp.v.R : 0;
+    for (auto &hp : plan.probs)
+        if (hp.v.D >= 8) hp.v.beside = large - hp.v.R;
     plan.status_off = take(256);
     plan.step_off = take(sizeof(StepState) * plan.probs.size());
     size_t acf_part = 0;
@@ -891,7 +895,7 @@ qst_status autotune_propose(qst_handle *h) {
         ProblemView &v = hp.v;
         if (v.D > 16 || (v.qr_passes != 0 && v.qr_passes != 3) || h->cfg.propose_threads != 0) continue;
         const int64_t blocks128 = (v.R + 128 / v.D - 1) / (128 / v.D);
-        if (blocks128 >= 2 * 5 * (int64_t)sms || propose_split(v, v.R)) continue;
+        if (blocks128 >= 2 * 5 * (int64_t)sms || propose_split(v, v.R, true)) continue;
         int best = 128;
         float best_ms = 0.0f;
         for (int threads : {128, 64, 32}) {
@@ -1399,7 +1403,7 @@ qst_status qst_diagnostics(qst_handle *h, int32_t problem, qst_diag *out, double
                                                                         : h->cfg.precision
                                                  : (int32_t)QST_PREC_FP32;
     out->propose_chains_per_cta =
-        (uint32_t)(v.D <= 16 ? (propose_split(v, v.R) ? 32 : v.propose_threads) / v.D : (v.D == 32 ? (v.qr_passes == 3 ? 2 : 4) : 1));
+        (uint32_t)(v.D <= 16 ? (propose_split(v, v.R, true) ? 32 : v.propose_threads) / v.D : (v.D == 32 ? (v.qr_passes == 3 ? 2 : 4) : 1));
     out->qr_passes = v.qr_passes;
     out->accept_chains_per_cta = (uint32_t)v.accept_cpc;
     if (st != QST_OK) return st;

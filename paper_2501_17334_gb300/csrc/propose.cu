@@ -1456,7 +1456,7 @@ cudaError_t launch_propose_pd(const ProblemView &p, int mode, uint32_t step, Ste
         // the CTA sizes the autotuner may pick are built for the default QR (3) and the
         // Hilbert-Schmidt prior (0); other settings run 128-thread CTAs
         if constexpr (PASSES == 3 && D >= 8) {
-            if (propose_split(p, rows)) return launch_propose_small<D, PASSES, 64, 2>(a, rows, s);
+            if (propose_split(p, rows, mode != MODE_EVAL)) return launch_propose_small<D, PASSES, 64, 2>(a, rows, s);
         }
         if constexpr (PASSES == 0 || PASSES == 3) {
             if (p.propose_threads == 32) return launch_propose_small<D, PASSES, 32>(a, rows, s);
@@ -1480,10 +1480,12 @@ cudaError_t launch_propose_d(const ProblemView &p, int mode, uint32_t step, Step
 // Two groups of lanes per chain (64-thread CTAs) at three and four qubits with the default QR and no
 // CTA size asked for, up to two warps per scheduler at four qubits and one at three.  us at one / two
 // groups: four qubits 64 chains 23.9 / 17.9, 1001 25.1 / 23.7, 2000 31.6 / 34.8; three qubits 64 chains
-// 11.8 / 10.5, 1000 12.5 / 9.8, 2000 11.9 / 12.7.
-bool propose_split(const ProblemView &p, int64_t rows) {
+// 11.8 / 10.5, 1000 12.5 / 9.8, 2000 11.9 / 12.7.  In a step the handle's other problems of that size run at
+// the same time and count as well, since the extra instructions then cost more than they shorten (277
+// four-qubit chains beside 2087: 54 us per step with one group, 58 with two).
+bool propose_split(const ProblemView &p, int64_t rows, bool step) {
     if (p.qr_passes != 3 || p.propose_fixed) return false;
-    return (p.D == 16 || p.D == 8) && rows <= 1216;
+    return (p.D == 16 || p.D == 8) && rows + (step ? p.beside : 0) <= 1216;
 }
 
 cudaError_t launch_propose(const ProblemView &p, int mode, uint32_t step, StepState *step_dev, const float *x_eval,

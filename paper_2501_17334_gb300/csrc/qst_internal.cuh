@@ -201,6 +201,7 @@ struct ProblemView {
                                  // (Hilbert-Schmidt prior, W = G)
     int propose_threads = 128;   // CTA size of the proposal kernel at D <= 16 (32, 64 or 128; autotuned)
     bool propose_fixed = false;  // that size was asked for
+    int64_t beside = 0;          // chains of the handle's other problems of three qubits or more
 };
 
 struct SamplerParams {
@@ -214,7 +215,8 @@ struct SamplerParams {
 // step_dev: when not null the step is the one after it (MODE_STEP) and is opened, else `step` is used
 cudaError_t launch_propose(const ProblemView &p, int mode, uint32_t step, StepState *step_dev, const float *x_eval, int64_t n_eval,
                            bool want_split, float *rho_norm_out, uint32_t *status, cudaStream_t s);
-bool propose_split(const ProblemView &p, int64_t rows);   // two groups of lanes per chain (32 / D chains per CTA)
+// two groups of lanes per chain (32 / D chains per CTA), in a step or in a call by itself
+bool propose_split(const ProblemView &p, int64_t rows, bool step);
 cudaError_t launch_project_fp32(const ProblemView &p, const float *A, int64_t rows, double *out_part,
                                 float *p_out, cudaStream_t s);
 // step_dev, MODE_STEP: the counter whose open step this closes

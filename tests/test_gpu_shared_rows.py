@@ -61,3 +61,17 @@ def test_many_step_launches_on_ill_conditioned_states(qst, cuda_ok, form, q, cha
     assert not np.array_equal(a["y"], x)   # some proposals were accepted
     many.close()
     plain.close()
+
+
+def test_groups_by_the_handles_problems(qst, cuda_ok):
+    """Two groups while all of a handle's larger problems together are few; the same chains in either handle."""
+    few, more = W.config_problem(4, num_chains=500), W.config_problem(4, num_chains=800)
+    small = W.config_problem(2, num_chains=3000)
+    kw = dict(precision=qst.PREC_PAULI, diag_chains=0)
+    with qst.Sampler([few, small], **kw) as a, qst.Sampler([few, more], **kw) as b:
+        assert a.diagnostics()["propose_chains_per_cta"] == 2
+        assert b.diagnostics()["propose_chains_per_cta"] in (2, 4, 8)   # (32 threads, 64 or 128: timed)
+        for s in (a, b):
+            s.run_chains(6)
+        x, y = a.get_state(0), b.get_state(0)
+        assert all(np.array_equal(x[k], y[k]) for k in x)
