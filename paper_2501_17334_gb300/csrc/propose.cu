@@ -126,13 +126,19 @@ __global__ void __launch_bounds__(THREADS, (GRP == 1 ? propose_ctas<D>() : 5) * 
         // lanes then read and write consecutive 16-byte pieces of y, and H's blocks reach the lanes that own
         // their columns through shared memory (area B where the refinement keeps H's columns
         // anyway, the Q planes otherwise).
+        // At D = 4 a block is its lane's column and needs neither (through shared memory the kernel took 30.6
+        // instead of 28.7 us for 65536 chains).
         constexpr int BPC = D / 4;   // blocks per column
-        auto stage = [&](float *plane_h, float *plane_q, int blk, float4 v) {
+        auto stage = [&](float *plane_h, float *plane_q, int blk, float4 v, float2 (&own)[D / 2]) {
             const int col = blk / BPC, r = blk % BPC;
-            if constexpr (PASSES == 3)
+            if constexpr (D == 4) {
+                own[0] = make_float2(v.x, v.y);
+                own[1] = make_float2(v.z, v.w);
+            } else if constexpr (PASSES == 3) {
                 *reinterpret_cast<float4 *>(plane_h + col * D + 4 * (r ^ hsw<D, QC>(col))) = v;
-            else
+            } else {
                 *reinterpret_cast<float4 *>(plane_q + col * QC + 4 * (r ^ qsw<D, QC>(col))) = v;
+            }
         };
 #pragma unroll 1
         for (int part = 0; part < 4; ++part) {
@@ -158,18 +164,20 @@ __global__ void __launch_bounds__(THREADS, (GRP == 1 ? propose_ctas<D>() : 5) * 
                     yn.w = __fmaf_rn(coef_y, y0[q].w, coef_eta * z3);
                     if (active) *reinterpret_cast<float4 *>(ydst + e0 + 4 * LPC * q) = yn;
                 }
-                if (part == 2) stage(hre, qre, l + LPC * q, yn);
-                if (part == 3) stage(him, qim, l + LPC * q, yn);
+                if (part == 2) stage(hre, qre, l + LPC * q, yn, hr);
+                if (part == 3) stage(him, qim, l + LPC * q, yn, hi);
             }
         }
-        __syncwarp();
-        if constexpr (PASSES == 3) {
-            load_column2<D>(hre + j * D, hr, hsw<D, QC>(j));
-            load_column2<D>(him + j * D, hi, hsw<D, QC>(j));
-        } else {
-            load_column2<D>(qre + j * QC, hr, qsw<D, QC>(j));
-            load_column2<D>(qim + j * QC, hi, qsw<D, QC>(j));
-            __syncwarp();   // (the sweep publishes its columns there)
+        if constexpr (D > 4) {
+            __syncwarp();
+            if constexpr (PASSES == 3) {
+                load_column2<D>(hre + j * D, hr, hsw<D, QC>(j));
+                load_column2<D>(him + j * D, hi, hsw<D, QC>(j));
+            } else {
+                load_column2<D>(qre + j * QC, hr, qsw<D, QC>(j));
+                load_column2<D>(qim + j * QC, hi, qsw<D, QC>(j));
+                __syncwarp();   // (the sweep publishes its columns there)
+            }
         }
     } else {
         // D == 2: each part is one Philox block shared by the two lanes; lane j takes pair j
@@ -206,7 +214,7 @@ __global__ void __launch_bounds__(THREADS, (GRP == 1 ? propose_ctas<D>() : 5) * 
         }
     }
 
-    if constexpr (PASSES == 3 && D < 4) {   // H's original columns, for the refinement after the sweep (above for D >= 4)
+    if constexpr (PASSES == 3 && D <= 4) {   // H's original columns, for the refinement after the sweep (above for D > 4)
         store_column2<D>(hre + j * D, hr, hsw<D, QC>(j));
         store_column2<D>(him + j * D, hi, hsw<D, QC>(j));
     }
