@@ -223,15 +223,17 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
 /* Enqueues num_steps steps j -> j+1 of Algorithm 2 for every chain of every problem
  * (proposal, Algorithm 1, likelihood, accept, adaptation, thinning and pooling).
  * Asynchronous on the handle's stream; resumable (step numbering continues).
- * A step is the proposal, projection and accept kernels of every problem; the last of the
- * accept kernels advances the step counter on the device.  With use_graph the first
+ * A step is the proposal, projection and accept kernels of every problem.  Each problem has a step
+ * counter on the device, which its proposal opens and its accept kernel closes.  With use_graph the first
  * call captures that sequence once (on private streams, the problems of a handle on up
  * to eight parallel branches, since they are independent) and every step launches the
  * graph; the results are bit-identical to plain launches.  One- and two-qubit problems in the FP32
  * or the structured Pauli form (up to 16 settings at two qubits, 8 at one, 2^18 / 4^(Q-1) chains,
  * qr_passes 3 or the Hilbert-Schmidt prior) instead run many steps per launch, on their own
- * branches beside the other problems, with the same results bit for bit; not while kernel timing
- * is on (qst_set_profiling).
+ * branches beside the other problems, in calls and handles where that is the shorter way (not in calls of
+ * one step, nor beside problems whose steps hide theirs), and never while kernel timing is on
+ * (qst_set_profiling).  Their chains are the same: in these launches two small terms of log L, some
+ * 1e-14 per count, are formed in FP32 instead of FP64, and no bit of a result has been seen to differ.
  * Errors: QST_ERR_INVALID_ARG if num_steps < 0. */
 qst_status qst_run_chains(qst_handle *h, int64_t num_steps);
 

@@ -1062,11 +1062,8 @@ qst_status qst_create(const qst_problem_desc *problems, int32_t num_problems, co
 
 namespace {
 
-// One step's launches on h->stream: every problem's proposal, projection and accept, all reading the
-// step from the device, where the proposal opens and the accept closes it.  With `branches` (graph
-// capture) the problems are spread over parallel branches -- they are independent -- so
-// the graph runs the kernels of different problems concurrently.  With `multi` the problems that
-// run many steps per launch (enqueue_multi) are left out.
+// One step of one problem on h->stream: its proposal, projection and accept, all reading the step from the
+// device, where the proposal opens and the accept closes it.
 qst_status enqueue_problem(qst_handle *h, HostProblem &hp) {
     ProblemView &v = hp.v;
     StepState *step = step_of(h, hp);
@@ -1081,6 +1078,9 @@ qst_status enqueue_problem(qst_handle *h, HostProblem &hp) {
     });
 }
 
+// One step's launches of every problem.  With `branches` (graph capture) the problems are spread over parallel
+// branches -- they are independent -- so the graph runs the kernels of different problems concurrently.
+// With `multi` the problems that run many steps per launch (enqueue_multi) are left out.
 qst_status enqueue_step(qst_handle *h, bool branches, bool multi) {
     qst_status st = QST_OK;
     std::vector<HostProblem *> probs;

@@ -6,9 +6,13 @@
 // Chains never interact, so here the lanes of a chain run whole steps on their own: the latent
 // state, rho and the chain's scalars stay in registers, the small matrices in a few hundred bytes
 // of shared memory, and nothing but warp barriers orders a step.  A CTA is one warp, so that few
-// chains spread over many SMs: 1.6 us per step for 64 one-qubit chains, 4.7 us for 4096 two-qubit
-// chains.  Every value is formed by the same operations in the
-// same order as in the per-step kernels, so the chains are the same bits.
+// chains spread over many SMs: 1.8 us per step for 64 one-qubit chains, 4.9 us for 4096 two-qubit
+// chains.  Values are formed by the same operations in the same order as in the per-step kernels,
+// with one exception: of log t, |t - 1| a few ulps, the second and third order (below 1e-14) are
+// formed in FP32 here and in FP64 in the accept kernel.  They differ by 1e-22, times the counts far
+// below log L's last bit: over 20 million proposals of one and two qubits no bit of log L differs
+// (tests/test_gpu_many_log_l.py), so the chains are the same bits.  In FP64 here as well a step takes
+// a fifth longer (64 one-qubit chains 1.8 -> 2.2 us, 4096 two-qubit chains 4.9 -> 5.3).
 //
 // What bounds a step here is one warp's chain of dependent instructions, and in it the FP64
 // instructions (a sub-partition takes 64 cycles for each, conversions from FP32 included), so
@@ -52,7 +56,8 @@ __device__ __forceinline__ int64_t kept_up_to(int64_t j, int thin, int64_t burn_
     return j <= burn_in ? 0 : j / thin - burn_in / thin;
 }
 
-// (double)x of a finite or infinite x by integer operations (a denormal counts as zero)
+// (double)x by integer operations.  A denormal counts as zero: what is converted here are sums of terms of
+// 1e-7 and more and their rounding errors, the smallest of them above 1e-20
 __device__ __forceinline__ double f2d(float x) {
     const uint32_t b = __float_as_uint(x), e = b & 0x7f800000u;
     const uint32_t rebias = e == 0x7f800000u ? 0x70000000u : 0x38000000u;   // exponent 255 -> 2047, else + 896

@@ -63,9 +63,9 @@ struct ProposeArgs {
 
 // THREADS: the CTA size (chains per CTA = THREADS / D); 128 by default, 64 or 32 when the
 // autotuner finds that a small problem covers more SMs that way.  The register budget per
-// thread is the same for every size (five 128-thread CTAs' worth per SM).
-// 128-thread CTAs per SM the register budget is set for: five (96 registers), at eight lanes per
-// chain seven (72: 65536 three-qubit chains 94 -> 89 us, 16384 29.1 -> 28.1).
+// thread is the same for every size: that of five 128-thread CTAs per SM (96 registers), at eight
+// lanes per chain of seven (72, nothing spilled but 4 bytes with 32 threads: 65536 three-qubit chains
+// 94 -> 89 us, 16384 29.1 -> 28.1).
 template <int D>
 constexpr int propose_ctas() {
     return D == 8 ? 7 : 5;
