@@ -100,6 +100,7 @@ struct HostProblem {
     ProblemView v{};
     int Q = 0, K = 0, KDmax = 0;
     int part_slots = 0;               // partial sums per chain the workspace holds (largest schedule)
+    int group_slots = 0;              // of them what the list kernel takes for all chains
     std::vector<int> group_choices;   // candidate ngroups values for the autotuner
     // QST_PREC_AUTO: the forms this problem's projection can take, and the tensor-core form's
     // column-group rule and candidates (kept while the structured Pauli form is in use)
@@ -484,7 +485,10 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
             if (fp32_lists(v)) count_list_rows(hp);
             v.ngroups = fp32_ngroups(v, v.R);
             const int nt = v.KD_pad / 128;
-            if (fp32_lists(v)) saved_slots = nt;
+            if (fp32_lists(v)) {   // (evaluation of fewer rows may take the list kernel where the chains do not)
+                saved_slots = nt;
+                hp.group_slots = fp32_list_groups(v, v.R);
+            }
             if (fp32_list_form(v, v.R)) {   // an even share for every SM: nothing to tune
                 hp.group_choices = {v.ngroups};
             } else {
@@ -492,7 +496,7 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
                 hp.group_choices.push_back(nt);
             }
         }
-        hp.part_slots = v.ngroups;
+        hp.part_slots = std::max(v.ngroups, hp.group_slots);
         for (int g : hp.group_choices) hp.part_slots = std::max(hp.part_slots, g);
         for (int g : hp.tc_group_choices) hp.part_slots = std::max(hp.part_slots, g);
         if (saved_slots > 0) hp.part_slots = std::max(hp.part_slots, saved_slots);

@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(SparseShape<D, C>::threads, 1) project_fp32_sp
     // There the deviance terms are added as the tiled kernel adds them -- one running Kahan sum per
     // four outcomes (packed here: outcomes u and u + 4), through the unit's two settings -- since
     // with few settings the order of that sum is the largest difference left between the two kernels
-    // (1e-9 of log L; at four qubits 4e-10).
+    // (1e-9 of log L).
     constexpr bool PAIR = D == 8;
     const int units = PAIR ? a.K / 16 * 8 + min(8, a.K % 16) : a.K;
     auto first_of = [&](int u) { return PAIR ? u / 8 * 16 + u % 8 : u; };
@@ -932,8 +932,12 @@ bool fp32_list_form(const ProblemView &p, int64_t rows) {
     return list <= (p.D == 8 ? 14.0 + 18.7 * waves : 13.0 + 43.5 * waves);
 }
 
+int fp32_list_groups(const ProblemView &p, int64_t rows) {
+    return sparse_groups(sparse_tiles(p, rows), sparse_ctas(p, rows));
+}
+
 int fp32_ngroups(const ProblemView &p, int64_t rows) {
-    if (fp32_list_form(p, rows)) return sparse_groups(sparse_tiles(p, rows), sparse_ctas(p, rows));
+    if (fp32_list_form(p, rows)) return fp32_list_groups(p, rows);
     // enough CTAs to fill the machine: split the columns when there are few row tiles
     const int64_t mt = (rows + BM - 1) / BM;
     const int nt = p.KD_pad / BN;

@@ -265,6 +265,7 @@ int fp32_ngroups(const ProblemView &p, int64_t rows);
 // the list kernel (else the tiled one), whether this size has them, the
 // floats, codes and lengths they take, and the kernel that makes them from P ([d][ld], device).
 bool fp32_list_form(const ProblemView &p, int64_t rows);
+int fp32_list_groups(const ProblemView &p, int64_t rows);   // partial sums per row of the list kernel
 bool fp32_lists(const ProblemView &p);
 size_t fp32_list_values(const ProblemView &p);
 size_t fp32_list_codes(const ProblemView &p);

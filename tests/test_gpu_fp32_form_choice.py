@@ -63,3 +63,24 @@ def test_a_handle_changes_with_the_rows(qst, cuda_ok):
                 _check(qst, prob, 4, s, n)
             s.run_chains(3)
             _check(qst, prob, 4, s, rows[0])
+
+
+def test_rows_close_to_the_chains(qst, cuda_ok):
+    """16384 chains run tiled in one column group, 12000 rows of them take the lists, over all SMs: the
+    projection of fewer rows is no slower than twice that of all."""
+    import torch
+    prob = W.random_basis_problem(4, 5, num_chains=16384)
+    with qst.Sampler(prob, diag_chains=0) as s:
+        assert s.diagnostics()["column_groups"] not in _list_groups(16384)
+        _check(qst, prob, 4, s, 12000)
+        s.set_profiling(True)
+        us = []
+        for n in (16384, 12000):
+            x = torch.from_numpy(W.latent_batch(n, 4, 3).astype(np.float32)).cuda()
+            s.evaluate(x)
+            s.kernel_time(qst.KERNEL_PROJECT, reset=True)
+            for _ in range(5):
+                s.evaluate(x)
+            ms, k = s.kernel_time(qst.KERNEL_PROJECT, reset=True)
+            us.append(ms / k * 1e3)
+        assert us[1] < 2 * us[0], us
