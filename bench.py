@@ -39,26 +39,33 @@ WORKLOAD = ("config 4: 4-qubit Pauli QST (D=16, 81 bases x 16 outcomes = 1296 pr
 # DRAM bytes per launch of each kernel from one ncu capture (bench.py --profile-case,
 # config 4 problem at `chains` chains, one pCN-step launch of the kernel), scaled to a launch
 # over the benchmark's chains in proportion to the chains processed.  The capture is only
-# used while the kernel's source file still has the recorded SHA-256.
+# used while every source file the kernel is built from is as it was: `sha256` is of their contents,
+# one after the other.
+CSRC = "paper_2501_17334_gb300/csrc/"
 NCU_TRAFFIC = {
     # profiles/propose_kernel_config4.md
-    "propose": {"source": "paper_2501_17334_gb300/csrc/propose.cu",
-                "sha256": "2fb35f57c9ef3a07e38ae82acda70f32930707cb1dfc3eec02eedc7c89bfc618",
-                "chains": 32768, "bytes": 137.376768e6 + 168.585472e6},
+    "propose": {"sources": [CSRC + f for f in ("propose.cu", "propose_dev.cuh", "f32x2.cuh", "log_poly.h",
+                                               "qst_internal.cuh")],
+                "sha256": "31de98d510cfda31f46c6a6d4966086a6de5bf161bdbfa03308315d7b7d01575",
+                "chains": 32768, "bytes": 137.366272e6 + 168.434944e6},
     # profiles/project_tc_kernel_config4.md
-    "project": {"source": "paper_2501_17334_gb300/csrc/project_tc.cu",
-                "sha256": "db5db012f46a894fd5b3793ee990c3d2d63468449643e6afb93cff51de19ec99",
-                "chains": 32768, "bytes": 51.39968e6 + 0.005376e6},
+    "project": {"sources": [CSRC + f for f in ("project_tc.cu", "f32x2.cuh", "log_poly.h", "qst_internal.cuh")],
+                "sha256": "3b33ac973a829547b3ce2b71a526f178355cc1bc5e75e93f6b8e04beafa59966",
+                "chains": 32768, "bytes": 51.399936e6 + 0.007680e6},
 }
 
-def _sha256(path):
-    with open(os.path.join(ROOT, path), "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()
+
+def _sha256(paths):
+    h = hashlib.sha256()
+    for path in paths:
+        with open(os.path.join(ROOT, path), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()
 
 
 def ncu_traffic(kernel, chains):
     rec = NCU_TRAFFIC.get(kernel)
-    if not rec or rec["bytes"] is None or rec["sha256"] != _sha256(rec["source"]):
+    if not rec or rec["bytes"] is None or rec["sha256"] != _sha256(rec["sources"]):
         return None
     return rec["bytes"] * chains / rec["chains"]
 

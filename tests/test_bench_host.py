@@ -4,6 +4,7 @@ the keys the benchmark's JSON line carries, even for runs short enough that the 
 initialisation, which every oracle run repeats, is comparable to the timed steps."""
 import json
 import os
+import re
 import subprocess
 import sys
 
@@ -32,3 +33,23 @@ def test_cpu_baseline_is_positive(oracle_mod, q):
     from paper_2501_17334_gb300 import workload as W
     r = bench.cpu_baseline(oracle_mod, W.config_problem(q), 0.5, label=f"{q}-qubit", max_steps=200)
     assert r["value"] > 0 and r["cores"] >= 1 and r["kind"] == "oracle"
+
+
+def test_traffic_records_cover_their_kernels_sources():
+    """A recorded DRAM traffic is keyed to the kernel's file and to every header of this repository it
+    includes, directly or not."""
+    sys.path.insert(0, ROOT)
+    import bench
+    csrc = os.path.join(ROOT, "paper_2501_17334_gb300", "csrc")
+
+    def included(name, seen):
+        if name not in seen and os.path.exists(os.path.join(csrc, name)):
+            seen.add(name)
+            for inc in re.findall(r'#include "([^"/]+)"', open(os.path.join(csrc, name)).read()):
+                included(inc, seen)
+        return seen
+    for kernel, top in (("propose", "propose.cu"), ("project", "project_tc.cu")):
+        rec = bench.NCU_TRAFFIC[kernel]
+        assert {os.path.basename(p) for p in rec["sources"]} == included(top, set())
+        assert rec["sha256"] == bench._sha256(rec["sources"])
+        assert bench.ncu_traffic(kernel, rec["chains"]) == rec["bytes"]
