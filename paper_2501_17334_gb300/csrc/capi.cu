@@ -295,14 +295,22 @@ void pauli_povms(int Q, std::vector<double> &re, std::vector<double> &im) {
 // The rows of P each setting's list will hold (those where one of its elements is not zero, or one)
 void count_list_rows(HostProblem &hp) {
     ProblemView &v = hp.v;
+    std::vector<int> used(hp.K, 0);
+    for (int r = 0; r < v.d; ++r) {
+        const float *row = hp.P32.data() + (size_t)r * v.KD_pad;
+        for (int k = 0; k < hp.K; ++k, row += v.D) {
+            uint32_t any = 0u;   // of the magnitudes' bits
+            for (int l = 0; l < v.D; ++l) {
+                uint32_t bits;
+                std::memcpy(&bits, row + l, sizeof bits);
+                any |= bits & 0x7fffffffu;
+            }
+            used[k] += any != 0u ? 1 : 0;
+        }
+    }
     v.sp_rows = 0;
     v.sp_most = 0;
-    for (int k = 0; k < hp.K; ++k) {
-        int n = 0;
-        for (int r = 0; r < v.d; ++r) {
-            const float *row = hp.P32.data() + (size_t)r * v.KD_pad + k * v.D;
-            n += std::any_of(row, row + v.D, [](float x) { return !(x == 0.0f); }) ? 1 : 0;
-        }
+    for (int n : used) {
         v.sp_rows += std::max(n, 1);
         v.sp_most = std::max(v.sp_most, std::max(n, 1));
     }
@@ -485,12 +493,13 @@ qst_status make_plan(const qst_problem_desc *probs_in, int32_t n, const qst_samp
             if (fp32_lists(v)) count_list_rows(hp);
             v.ngroups = fp32_ngroups(v, v.R);
             const int nt = v.KD_pad / 128;
-            if (fp32_lists(v)) {   // (evaluation of fewer rows may take the list kernel where the chains do not)
+            if (fp32_lists(v)) {
+                // the list kernel gives every SM an even share, and where the tiled one is taken its rule's
+                // groups make whole waves: nothing to tune.  (Evaluation of fewer rows may take the list
+                // kernel where the chains do not.)
+                hp.group_choices = {v.ngroups};
                 saved_slots = nt;
                 hp.group_slots = fp32_list_groups(v, v.R);
-            }
-            if (fp32_list_form(v, v.R)) {   // an even share for every SM: nothing to tune
-                hp.group_choices = {v.ngroups};
             } else {
                 for (int g = 1; g < nt; g *= 2) hp.group_choices.push_back(g);
                 hp.group_choices.push_back(nt);
@@ -610,6 +619,7 @@ struct qst_handle {
         int64_t kernels = 0;                 // kernel launches one replay performs
     };
     StepGraph steps_graph, single_graph;     // a step of the problems that go step by step, and of all of them
+    bool single_before = false;              // problems of many-step launches went step by step in a call
     int64_t steps_done = 0;
     int64_t kept = 0;
     int64_t launches = 0;
@@ -1273,13 +1283,19 @@ qst_status qst_run_chains(qst_handle *h, int64_t num_steps) {
     if (!h->prof)
         for (auto &hp : h->plan.probs)
             if (fused_supported(hp.v)) multi.push_back(&hp);
+    const bool all_multi = multi.size() == h->plan.probs.size();
     const bool single = !multi.empty() && !multi_step_pays(h, multi, num_steps);   // all step by step
     if (single) multi.clear();
     const bool steps = multi.size() < h->plan.probs.size();   // some problems go step by step
     qst_handle::StepGraph *graph = nullptr;
     if (h->cfg.use_graph && !h->prof && steps) {
         graph = single ? &h->single_graph : &h->steps_graph;
-        if (!graph->exec) {
+        // (where such a call is an exception the graph is not worth its capture: the first goes by plain launches)
+        const bool first = single && all_multi && !h->single_before;
+        h->single_before = h->single_before || single;
+        if (first) {
+            graph = nullptr;
+        } else if (!graph->exec) {
             qst_status st = build_step_graph(h, !multi.empty(), *graph);
             if (st != QST_OK) return st;
         }

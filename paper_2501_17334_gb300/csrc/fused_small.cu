@@ -200,7 +200,9 @@ __global__ void __launch_bounds__(kWarp, kMinCtas) fused_small_kernel(const __gr
     constexpr int chains = kWarp / LPC;   // of this CTA
     const int64_t c = (int64_t)blockIdx.x * chains + g;
     const bool active = c < p.R;
-    const int64_t cc = active ? c : 0;   // (an idle group repeats chain 0 and writes nothing)
+    // an idle group repeats the last chain, which is of this warp, and writes nothing (another warp's chain
+    // could be written back while it is read)
+    const int64_t cc = active ? c : p.R - 1;
     float *sm = smem + g * F::stride;
     float *qre = sm, *qim = sm + D * QC;
     float2 *wsm = reinterpret_cast<float2 *>(sm);
