@@ -1211,7 +1211,7 @@ double step_us(const ProblemView &v) {
 // join: two steps of eight two-qubit problems 65 instead of 54, three 73 instead of 80.
 //   Beside problems that go step by step, a small one on a branch of its own in the step graph costs nothing,
 // while its launches are extra and their CTAs slow the others down: one of 4096 two-qubit chains beside 16384
-// three-qubit ones 51.6 us per step instead of 48.3, six mixed problems two steps 136 instead of 93.  There the
+// three-qubit ones 51.6 us per step instead of 48.5, six mixed problems two steps 134 instead of 88.  There the
 // launches pay where the small problems lengthen the graph's branches (30 one-qubit problems and a four-qubit
 // one 38 us per step instead of 75) or are large and spare the chip work (65536 two-qubit chains in the FP32 form
 // beside three-qubit ones 60 instead of 76; in the Pauli form they spare none).
